@@ -61,6 +61,20 @@ __device__ __forceinline__ void ds_mul(float ah, float al, float bh, float bl, f
   l = __fsub_rn(t, __fsub_rn(h, p));
 }
 
+// (s1, s2, s3) += v: two chained TwoSums and an addition, so the unevaluated
+// sum s1 + s2 + s3 keeps about 72 bits, more than an FP64 sum of the same
+// FP32 terms.  13 FP32 operations a term, where the FP64 sum takes a
+// conversion and an addition on a pipe 64 times narrower.
+__device__ __forceinline__ void ts_add(float v, float& s1, float& s2, float& s3) {
+  const float a = __fadd_rn(s1, v), ab = __fsub_rn(a, s1);
+  const float e1 = __fadd_rn(__fsub_rn(s1, __fsub_rn(a, ab)), __fsub_rn(v, ab));
+  const float b = __fadd_rn(s2, e1), bb = __fsub_rn(b, s2);
+  const float e2 = __fadd_rn(__fsub_rn(s2, __fsub_rn(b, bb)), __fsub_rn(e1, bb));
+  s1 = a;
+  s2 = b;
+  s3 = __fadd_rn(s3, e2);
+}
+
 // An FP64 value as a double-single pair.
 __device__ __forceinline__ void ds_split(double v, float& h, float& l) {
   h = __double2float_rn(v);
