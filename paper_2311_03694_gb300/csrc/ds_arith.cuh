@@ -75,6 +75,23 @@ __device__ __forceinline__ void ts_add(float v, float& s1, float& s2, float& s3)
   s3 = __fadd_rn(s3, e2);
 }
 
+// An FP32 value as FP64 and an FP64 value rounded (to nearest even) to FP32,
+// on the integer pipe: a conversion instruction takes a slot of the FP64
+// pipe, as long as some thirty integer operations.  Zeros, subnormals,
+// infinities and NaNs, and what rounds to them, take the instruction.
+__device__ __forceinline__ double f2d_int(float x) {
+  const unsigned int v = (unsigned int)__float_as_int(x), mag = v & 0x7fffffffu;
+  if (mag - 0x00800000u >= 0x7f000000u) return (double)x;
+  return __hiloint2double((int)((v & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(v << 29));
+}
+__device__ __forceinline__ float d2f_int(double x) {
+  const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);
+  if (((hi >> 20) & 0x7ffu) - 897u >= 254u) return __double2float_rn(x);
+  unsigned int mag = (__funnelshift_l(lo, hi, 3) - 0x40000000u) & 0x7fffffffu;  // the 29 low bits cut off
+  mag += ((lo & 0x1fffffffu) + 0x0fffffffu + (mag & 1u)) >> 29;
+  return __int_as_float((int)((hi & 0x80000000u) | mag));
+}
+
 // An FP64 value as a double-single pair.
 __device__ __forceinline__ void ds_split(double v, float& h, float& l) {
   h = __double2float_rn(v);

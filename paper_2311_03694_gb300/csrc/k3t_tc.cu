@@ -781,7 +781,8 @@ __global__ void __launch_bounds__(K3T_THREADS, 1)
           if (on[e]) {
             const double* h = st.hist + bq[e] * st.hist_stride;
             const int m0 = (int)(lq[e] % 3);
-            for (int q = 0; q < pp.kf.s2; ++q) nl[e] += (double)pp.kf.d2[((int64_t)q * pp.kf.bp + b) * n + iq[e]];
+            nl[e] = f2d_int(pp.kf.d2[(int64_t)b * n + iq[e]]);
+            for (int q = 1; q < pp.kf.s2; ++q) nl[e] += f2d_int(pp.kf.d2[((int64_t)q * pp.kf.bp + b) * n + iq[e]]);
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
               const int m = m0 - q < 0 ? m0 - q + 3 : m0 - q;
@@ -797,25 +798,16 @@ __global__ void __launch_bounds__(K3T_THREADS, 1)
         for (int e = 0; e < 4; ++e) {
           if (!on[e]) continue;
           // the plain diagonal step (step_elem with PLAIN), from the loaded operands
-          const int k = kq[e];
-          double ext = 0.0, bdf = 0.0;
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            if (q < k) {
-              const double gq = q == 0 ? nl[e] : nq[e][q];
-              ext = fma(c_alpha[k - 1][q], gq, ext);
-              bdf = fma(st.bdt[k - 1][q], uq[e][q], bdf);
-            }
-          }
-          const double un = -(ext + bdf) * hd[e];
+          const double ge[3] = {nl[e], nq[e][1], nq[e][2]};
+          const double un = step_plain_elem(st.bdt[kq[e] - 1], kq[e], uq[e], ge, hd[e]);
           double* h = st.hist + bq[e] * st.hist_stride;
           h[(3 + lq[e] % 3) * n + iq[e]] = nl[e];
           h[((lq[e] + 1) % 3) * n + iq[e]] = un;
-          const float v = __double2float_rn(un);
+          const float v = d2f_int(un);
           const __nv_bfloat16 hi = __float2bfloat16_rn(v);
           xh[(int64_t)bq[e] * pp.np + iq[e]] = hi;
           xl[(int64_t)bq[e] * pp.np + iq[e]] = __float2bfloat16_rn(v - __bfloat162float(hi));
-          if (((__double_as_longlong(un) >> 52) & 0x7FF) == 0x7FF) report_nonfinite(st, bq[e]);
+          if (step_is_bad(un)) report_nonfinite(st, bq[e]);
         }
       }
     }

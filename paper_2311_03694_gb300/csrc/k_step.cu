@@ -62,8 +62,118 @@ __global__ void __launch_bounds__(STEP_MC_THREADS) k_step_diag_mc(const StepArgs
                        [] { __syncthreads(); }, sh, &bad, &last);
 }
 
+// The plain diagonal step (step_plain) of large batches: a block of 256
+// threads steps EPT x 256 elements of one trajectory, each thread with the
+// loads of its EPT elements in flight together.  FUSE: 0 n^l from the
+// history ring, 2 the K3T expansion partials with the new state's BF16 hi/lo
+// rows written (as step_mc_block).  The same element arithmetic, so the same
+// bits, as the kernel above.
+//
+// Six FP64 operations an element (and one per partial after the first) and
+// some 68 bytes are what it has to do: at two FP64 operations a clock and SM
+// the pipe stays the bound while the state lies in L2.  A row of up to 1024
+// elements is one block, which needs no arrival counter to advance the step
+// count.  1024 trajectories of n = 1024, cold caches (ncu): 24.7 us with K3T's
+// two partials and 20.9 us without, against 34.5 and 28.2 us with one element
+// a thread and eight operations (13 with the conversions).
+constexpr int STEP_PLAIN_THREADS = 256;
+template <int FUSE, int EPT>
+__global__ void __launch_bounds__(STEP_PLAIN_THREADS) k_step_plain(const StepArgs a,
+                                                                   const K3TStepFuse kf) {
+  __shared__ int last;
+  const int b = blockIdx.y, tid = threadIdx.x;
+  if (a.active && !a.active[b]) return;  // uniform over the block
+  const int n = (int)a.n;
+  const int64_t l = a.taken[b];
+  const int k = (int)(l + 1 < a.order ? l + 1 : a.order);
+  const int m0 = (int)(l % 3);
+  double* h = a.hist + b * a.hist_stride;
+  const double* hd = a.hdiag[k - 1];
+  double u[EPT][3], g[EPT][3], d[EPT];
+  const int i0 = blockIdx.x * (STEP_PLAIN_THREADS * EPT) + tid;
+#pragma unroll
+  for (int e = 0; e < EPT; ++e) {
+    const int i = i0 + e * STEP_PLAIN_THREADS;
+    d[e] = 0.0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int m = m0 - q < 0 ? m0 - q + 3 : m0 - q;
+      u[e][q] = g[e][q] = 0.0;
+      if (i < n && q < k) {
+        u[e][q] = h[m * n + i];
+        if (q > 0 || FUSE == 0) g[e][q] = h[(3 + m) * n + i];
+      }
+    }
+    if (i < n) d[e] = hd[i];
+  }
+  if constexpr (FUSE == 2) {
+    const float* p = kf.d2 + (int64_t)b * n;
+    const int64_t split = kf.bp * (int64_t)n;
+    float w[EPT];
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) w[e] = i0 + e * STEP_PLAIN_THREADS < n ? p[i0 + e * STEP_PLAIN_THREADS] : 0.f;
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) g[e][0] = f2d_int(w[e]);
+    for (int s = 1; s < kf.s2; ++s) {
+      p += split;
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) w[e] = i0 + e * STEP_PLAIN_THREADS < n ? p[i0 + e * STEP_PLAIN_THREADS] : 0.f;
+#pragma unroll
+      for (int e = 0; e < EPT; ++e) g[e][0] += f2d_int(w[e]);
+    }
+  }
+  int bad = 0;
+  const int mn = m0 == 2 ? 0 : m0 + 1;  // (l + 1) mod 3
+#pragma unroll
+  for (int e = 0; e < EPT; ++e) {
+    const int i = i0 + e * STEP_PLAIN_THREADS;
+    if (i >= n) continue;
+    const double un = step_plain_elem(a.bdt[k - 1], k, u[e], g[e], d[e]);
+    bad |= step_is_bad(un);
+    if constexpr (FUSE == 2) {
+      h[(3 + m0) * n + i] = g[e][0];
+      const float v = d2f_int(un);
+      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
+      static_cast<__nv_bfloat16*>(kf.xh)[(int64_t)b * kf.np + i] = hi;
+      static_cast<__nv_bfloat16*>(kf.xl)[(int64_t)b * kf.np + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
+    }
+    h[mn * n + i] = un;
+  }
+  bad = __syncthreads_or(bad);  // also: every thread has read the step count
+  if (tid == 0 && bad) report_nonfinite(a, b);
+  if (gridDim.x == 1) {
+    if (tid == 0) step_done(a, b, l);
+    return;
+  }
+  if (tid == 0) last = atomicAdd(&a.cnt[b], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (last && tid == 0) {
+    step_done(a, b, l);
+    a.cnt[b] = 0u;
+  }
+}
+
+// The plain step of `batch` trajectories, or false when the kernel of the
+// general case is the better one: with fewer than about two blocks an SM the
+// short blocks of one element a thread spread further.
+template <int FUSE>
+static bool step_plain_launch(const StepArgs& a, const K3TStepFuse& f, cudaStream_t s) {
+  const int64_t per = a.n <= 256 ? 256 : a.n <= 512 ? 512 : 1024;
+  const int64_t blocks = (a.n + per - 1) / per;
+  if (!step_plain(a) || blocks * a.batch < 256 || a.batch > 65535) return false;
+  const dim3 grid((unsigned)blocks, (unsigned)a.batch);
+  if (per == 256)
+    k_step_plain<FUSE, 1><<<grid, STEP_PLAIN_THREADS, 0, s>>>(a, f);
+  else if (per == 512)
+    k_step_plain<FUSE, 2><<<grid, STEP_PLAIN_THREADS, 0, s>>>(a, f);
+  else
+    k_step_plain<FUSE, 4><<<grid, STEP_PLAIN_THREADS, 0, s>>>(a, f);
+  return true;
+}
+
 cudaError_t step_diag_mc_launch(const StepArgs& a, int step_index, const K1Plan* k1, const K1Args* k1a, int b0, int nb,
                                 int nbk, cudaStream_t s) {
+  if (!k1 && b0 == 0 && nb == a.batch && step_plain_launch<0>(a, K3TStepFuse{}, s)) return cudaGetLastError();
   dim3 grid((unsigned)a.nblk, (unsigned)nb);
   K1Plan pl{};
   K1Args ka{};
@@ -78,6 +188,7 @@ cudaError_t step_diag_mc_launch(const StepArgs& a, int step_index, const K1Plan*
 
 static cudaError_t step_diag_mc_fused(const StepArgs& a, int step_index, int fuse, const K3TStepFuse& f,
                                       cudaStream_t s) {
+  if (fuse == 2 && step_plain_launch<2>(a, f, s)) return cudaGetLastError();
   dim3 grid((unsigned)a.nblk, (unsigned)a.batch);
   if (step_plain(a))
     k_step_diag_mc<true><<<grid, STEP_MC_THREADS, 0, s>>>(a, step_index, K1Plan{}, K1Args{}, fuse, 0, 1, f);

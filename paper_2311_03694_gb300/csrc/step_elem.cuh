@@ -19,16 +19,37 @@ static __constant__ double c_alpha[3][3] = {
     {3.0, -3.0, 1.0},
 };
 
+// EXTk of the newest k advection terms, g[0] the newest: g0, 2 g0 - g1 or
+// 3 (g0 - g1) + g2, in at most two FP64 operations.
+__device__ __forceinline__ double step_ext(int k, const double (&g)[3]) {
+  return k == 1 ? g[0] : k == 2 ? fma(2.0, g[0], -g[1]) : fma(3.0, __dsub_rn(g[0], g[1]), g[2]);
+}
+
+// u^{l+1}_i of the plain diagonal step (identity mass): the BDF terms chained
+// onto the extrapolation, six FP64 operations at order 3.
+__device__ __forceinline__ double step_plain_elem(const double (&bdt)[3], int k, const double (&u)[3],
+                                                  const double (&g)[3], double hd) {
+  double y = step_ext(k, g);
+  if (k == 3) y = fma(bdt[2], u[2], y);
+  if (k >= 2) y = fma(bdt[1], u[1], y);
+  y = fma(bdt[0], u[0], y);
+  return __dmul_rn(-y, hd);
+}
+
+__device__ __forceinline__ int step_is_bad(double un) {  // inf or NaN, from the exponent bits
+  return ((__double_as_longlong(un) >> 52) & 0x7FF) == 0x7FF;
+}
+
 // One element of the diagonal step: u^{l+1}_i from the history and n^l_i = nl.
 // FP64 runs at about two operations per clock per SM on this part, so the
 // terms of absent operators (mass, linear, forcing: null pointers, uniform
 // branches) are skipped, beta/dt comes from the host, the energy and
 // invariant terms are formed only when `sums` is set, and finiteness is
-// read from the exponent bits: about eight FP64 operations per element in
-// the common case.  PLAIN (no mass, linear or forcing term, no sums) removes
+// read from the exponent bits: six FP64 operations per element in the common
+// case.  PLAIN (no mass, linear or forcing term, no sums) removes
 // those terms at compile time: a runtime test still issues its predicated
 // FP64 instructions, which measured ~26 FP64 instructions per element on the
-// batched step against the 8 of the plain arithmetic.
+// batched step.
 template <bool PLAIN = false>
 __device__ __forceinline__ double step_elem(const StepArgs& a, double* h, int64_t n, int64_t l, int k, int64_t i,
                                             double nl, double& e_part, double& i_part, int& bad, bool sums = true) {
@@ -38,26 +59,27 @@ __device__ __forceinline__ double step_elem(const StepArgs& a, double* h, int64_
   const double ld = lin ? a.lin_diag[i] : 0.0;
   const double f = frc ? a.forcing[i] : 0.0;
   const int m0 = (int)(l % 3);
-  double ext = 0.0, bdf = 0.0, u0 = 0.0;
+  double u[3] = {0.0, 0.0, 0.0}, g[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     if (q < k) {
       const int m = m0 - q < 0 ? m0 - q + 3 : m0 - q;
-      const double uq = h[m * n + i];
-      double g = q == 0 ? nl : h[(3 + m) * n + i];
-      if (q == 0) u0 = uq;
-      if (lin) g = fma(ld, uq, g);
-      if (frc) g += f;
-      ext = fma(c_alpha[k - 1][q], g, ext);
-      bdf = fma(a.bdt[k - 1][q], uq, bdf);
+      u[q] = h[m * n + i];
+      g[q] = q == 0 ? nl : h[(3 + m) * n + i];
+      if (lin) g[q] = fma(ld, u[q], g[q]);
+      if (frc) g[q] += f;
     }
   }
   double un, mb = 1.0;
   if (mass) {
     mb = a.mass_diag[i];
-    un = fma(-mb, bdf, -ext) * a.hdiag[k - 1][i];
+    double bdf = 0.0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (q < k) bdf = fma(a.bdt[k - 1][q], u[q], bdf);
+    un = fma(-mb, bdf, -step_ext(k, g)) * a.hdiag[k - 1][i];
   } else {
-    un = -(ext + bdf) * a.hdiag[k - 1][i];
+    un = step_plain_elem(a.bdt[k - 1], k, u, g, a.hdiag[k - 1][i]);
   }
   e_part = 0.0;
   i_part = 0.0;
@@ -65,9 +87,9 @@ __device__ __forceinline__ double step_elem(const StepArgs& a, double* h, int64_
     // explicit roundings: the products must not contract into the caller's
     // sums (FMA), whose form would then depend on the kernel inlining them
     e_part = mass ? __dmul_rn(__dmul_rn(mb, un), un) : __dmul_rn(un, un);
-    i_part = __dmul_rn(u0, nl);
+    i_part = __dmul_rn(u[0], nl);
   }
-  bad = ((__double_as_longlong(un) >> 52) & 0x7FF) == 0x7FF;  // inf or NaN
+  bad = step_is_bad(un);
   h[((l + 1) % 3) * n + i] = un;
   return un;
 }

@@ -99,8 +99,8 @@ __device__ __forceinline__ void step_mc_block(const StepArgs& a, int step_index,
       }
     } else if (fuse == 2) {
       // expansion splits in split order, FP64
-      double sum = 0.0;
-      for (int q = 0; q < kf.s2; ++q) sum += (double)kf.d2[((int64_t)q * kf.bp + b) * n + i];
+      double sum = f2d_int(kf.d2[(int64_t)b * n + i]);
+      for (int q = 1; q < kf.s2; ++q) sum += f2d_int(kf.d2[((int64_t)q * kf.bp + b) * n + i]);
       h[(3 + l % 3) * n + i] = sum;
       nl = sum;
     } else if (fuse) {
@@ -128,7 +128,7 @@ __device__ __forceinline__ void step_mc_block(const StepArgs& a, int step_index,
       static_cast<float*>(kf.xh)[i * kf.np + b] = hi;  // planes [i][b]
       static_cast<float*>(kf.xl)[i * kf.np + b] = lo;
     } else if (fuse == 2) {
-      const float v = __double2float_rn(un);
+      const float v = d2f_int(un);
       const __nv_bfloat16 hi = __float2bfloat16_rn(v);
       static_cast<__nv_bfloat16*>(kf.xh)[(int64_t)b * kf.np + i] = hi;
       static_cast<__nv_bfloat16*>(kf.xl)[(int64_t)b * kf.np + i] = __float2bfloat16_rn(v - __bfloat162float(hi));
