@@ -572,41 +572,67 @@ __global__ void k2p_prep_kernel(const K2PDev p, float* uf, __nv_bfloat16* uh, __
 // each group summed in a fixed order in FP32 (the partials are FP32 sums
 // already; FP64 adds run at about two per clock per SM on this part), the
 // two totals subtracted in FP64.
-__global__ void k2p_finish_kernel(const K2PDev p, double* c, int64_t c_stride, double* hist, const int64_t* taken,
-                                  int64_t hist_stride, const int32_t* active, int batch) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)batch * p.n) return;
-  const int64_t k = t / batch, b = t - k * batch;  // consecutive threads: consecutive b
-  if (active && !active[b]) return;
-  const int ct = (int)(b / p.btile), bl = (int)(b - (int64_t)ct * p.btile);
-  float sd = 0.f, sm = 0.f;
-  for (int pb = 0; pb < p.pblks; ++pb) sd += p.cdp[((int64_t)pb * p.n + k) * p.bp + b];
-  // window row w of tile (range r, block pb) holds the mirrored entries of
-  // k = (r m + 1 + 128 pb + w) mod n
-  for (int pb = 0; pb < p.pblks; ++pb) {
-    const int64_t x = ((k - 1 - (int64_t)pb * 128) % p.n + p.n) % p.n;
-    auto add = [&](int r) {
-      int64_t w = x - (int64_t)r * p.m;
-      if (w < 0) w += p.n;
-      const float* e = p.ep + ((int64_t)(r * p.pbs + pb) * p.col_tiles + ct) * p.wrows * p.btile + bl;
-      for (; w < p.wrows; w += p.n) sm += e[w * p.btile];
-    };
-    if (p.n <= p.wrows) {
-      for (int r = 0; r < p.ranges; ++r) add(r);
-    } else {
-      // w = x - r m for r m <= x, w = x - r m + n for r m > x; at most one row per tile
-      const int rhi = (int)(x / p.m);
-      const int rlo = x - p.wrows < 0 ? 0 : (int)((x - p.wrows) / p.m) + 1;
-#pragma unroll 4
-      for (int r = rlo; r <= rhi; ++r) add(r);
-      const int64_t y = x + p.n - p.wrows;
-      int r2 = y < 0 ? 0 : (int)(y / p.m) + 1;
-      if (r2 < rhi + 1) r2 = rhi + 1;
-      for (int r = r2; r < p.ranges; ++r) add(r);
+//
+// A block takes 16 test indices of 32 trajectories: a warp reads one test
+// index's 32 trajectories (128-byte lines), the totals turn through shared
+// memory and the rows of c are written 128 bytes at a time, with 32-bit index
+// arithmetic and independent loads (n = 1024, 1024 trajectories: 79.7 us
+// against 96.4).  Reading the 123 MB of partial sums once is its floor (18 us).
+constexpr int K2PF_K = 16, K2PF_B = 32, K2PF_WARPS = 8;
+__global__ void __launch_bounds__(32 * K2PF_WARPS)
+    k2p_finish_kernel(const K2PDev p, double* c, int64_t c_stride, double* hist, const int64_t* taken,
+                      int64_t hist_stride, const int32_t* active, int batch) {
+  __shared__ double sh[K2PF_B][K2PF_K + 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = (int)p.n, m = p.m, wrows = p.wrows;
+  const int k0 = blockIdx.x * K2PF_K, b0 = blockIdx.y * K2PF_B, b = b0 + lane;
+  const int ct = b / p.btile, bl = b - ct * p.btile;
+  const int64_t tile = (int64_t)wrows * p.btile;
+  for (int kq = warp; kq < K2PF_K; kq += K2PF_WARPS) {
+    const int k = k0 + kq;
+    if (k >= n || b >= batch) continue;
+    float sd = 0.f, sm = 0.f;
+    for (int pb = 0; pb < p.pblks; ++pb) sd += p.cdp[((int64_t)pb * n + k) * p.bp + b];
+    // window row w of tile (range r, block pb) holds the mirrored entries of
+    // k = (r m + 1 + 128 pb + w) mod n
+    int x = k > 0 ? k - 1 : n - 1;  // (k - 1 - 128 pb) mod n
+    for (int pb = 0; pb < p.pblks; ++pb) {
+      const float* base = p.ep + ((int64_t)pb * p.col_tiles + ct) * tile + bl;
+      const int64_t rstep = (int64_t)p.pbs * p.col_tiles * tile;  // from one range's tile to the next
+      if (n <= wrows) {  // the window wraps: a tile may hold several rows of k
+        for (int r = 0; r < p.ranges; ++r) {
+          int w = x - r * m;
+          if (w < 0) w += n;
+          const float* e = base + r * rstep;
+          for (; w < wrows; w += n) sm += e[(int64_t)w * p.btile];
+        }
+      } else {
+        // w = x - r m for r m <= x, w = x - r m + n for r m > x; at most one
+        // row per tile, `step` values apart, so the loads are independent
+        const int64_t step = rstep - (int64_t)m * p.btile;
+        const int rhi = x / m;
+        const int rlo = x - wrows < 0 ? 0 : (x - wrows) / m + 1;
+        const float* e = base + rlo * rstep + (int64_t)(x - rlo * m) * p.btile;
+#pragma unroll 8
+        for (int r = rlo; r <= rhi; ++r, e += step) sm += *e;
+        const int y = x + n - wrows;
+        int r2 = y < 0 ? 0 : y / m + 1;
+        if (r2 < rhi + 1) r2 = rhi + 1;
+        e = base + r2 * rstep + (int64_t)(x + n - r2 * m) * p.btile;
+        for (int r = r2; r < p.ranges; ++r, e += step) sm += *e;
+      }
+      x -= 128 % n;
+      if (x < 0) x += n;
     }
+    sh[lane][kq] = (double)sd - (double)sm;
   }
-  double* dst = taken ? hist + b * hist_stride + (3 + taken[b] % 3) * p.n : c + b * c_stride;
-  dst[k] = (double)sd - (double)sm;
+  __syncthreads();
+  for (int t = threadIdx.x; t < K2PF_K * K2PF_B; t += 32 * K2PF_WARPS) {
+    const int64_t k = k0 + t % K2PF_K, bt = b0 + t / K2PF_K;
+    if (k >= n || bt >= batch || (active && !active[bt])) continue;
+    double* dst = taken ? hist + bt * hist_stride + (3 + taken[bt] % 3) * p.n : c + bt * c_stride;
+    dst[k] = sh[t / K2PF_K][t % K2PF_K];
+  }
 }
 
 // ------------------------------------------------------------------- host
@@ -816,9 +842,9 @@ cudaError_t k2p_launch(const K2PPlan& p, const CUtensorMap* tmap, const K2Args& 
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (a.ev1) prof_record(a.ev1, s);
-  const int64_t red = (int64_t)a.batch * p.n;
-  k2p_finish_kernel<<<(unsigned)((red + 255) / 256), 256, 0, s>>>(d, a.c, a.c_stride, a.hist, a.taken,
-                                                                  a.hist_stride, a.active, a.batch);
+  const dim3 fin((unsigned)((p.n + K2PF_K - 1) / K2PF_K), (unsigned)((a.batch + K2PF_B - 1) / K2PF_B));
+  k2p_finish_kernel<<<fin, 32 * K2PF_WARPS, 0, s>>>(d, a.c, a.c_stride, a.hist, a.taken, a.hist_stride, a.active,
+                                                    a.batch);
   return cudaGetLastError();
 }
 
