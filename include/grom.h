@@ -86,7 +86,10 @@ typedef int32_t grom_status;
  * stores zero there).  The other entries follow from C_ijk = -C_kji, so
  *   c_i = sum_j u_j [ sum_d C_{i,j,i+d} u_{i+d} - sum_d C_{i-d,j,i} u_{i-d} ]
  * (indices mod n) is the same contraction as the dense one.  This halves the
- * bytes and the multiply-adds of the streaming contraction.
+ * bytes and the multiply-adds of the streaming contraction.  With F64 and
+ * F32X2 storage the full form keeps n^3 / 3 values instead, sums
+ * C_pqm + C_pmq for p, q < m (c depends on the entries through those sums
+ * only), each formed in FP64 and rounded once.
  * The caller's tensor must be skew to rounding.  While uploading, the library
  * forms the probe sum_ijk x_i y_j x_k C_ijk for two seeded +-1 vector pairs
  * (zero for a skew tensor, about ||sym(C)||_F otherwise) and rejects the

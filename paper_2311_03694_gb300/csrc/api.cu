@@ -125,8 +125,9 @@ static grom_status upload_rows_packed(grom_rom* r, const double* src, int64_t i0
     cudaError_t e = cudaMemcpyAsync(stage, src + (a - i0) * per_i, (size_t)(cnt * per_i * 8), cudaMemcpyDefault, r->stream);
     if (e == cudaSuccess) e = skew_probe_launch(stage, cnt * m, n, m, a, r->probe, r->stream);
     if (e == cudaSuccess)
-      e = convert_rows_packed_launch(stage, cnt * m, n, m, a, r->k1.lp, r->storage, r->op + a * m * r->k1.row_bytes,
-                                     r->stream);
+      e = r->folded ? k1t_convert(r->k1t, stage, a, cnt, r->op, r->stream)
+                    : convert_rows_packed_launch(stage, cnt * m, n, m, a, r->k1.lp, r->storage,
+                                                 r->op + a * m * r->k1.row_bytes, r->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(r->stream);
     if (e != cudaSuccess) {
       cudaFree(stage);
@@ -159,8 +160,9 @@ static grom_status upload_augmented_full(grom_rom* r, const double* src, std::ve
     if (e == cudaSuccess && packed) {
       e = skew_probe_launch(core, cnt * n, n, n, a, r->probe, r->stream);
       if (e == cudaSuccess)
-        e = convert_rows_packed_launch(core, cnt * n, n, n, a, r->k1.lp, r->storage, r->op + a * n * r->k1.row_bytes,
-                                       r->stream);
+        e = r->folded ? k1t_convert(r->k1t, core, a, cnt, r->op, r->stream)
+                      : convert_rows_packed_launch(core, cnt * n, n, n, a, r->k1.lp, r->storage,
+                                                   r->op + a * n * r->k1.row_bytes, r->stream);
     } else if (e == cudaSuccess) {
       e = convert_rows_launch(core, cnt * n, n, r->np, r->storage, r->op + a * n * r->k1.row_bytes, r->stream);
     }
@@ -218,7 +220,7 @@ static void rom_free(grom_rom* r) {
                   r->lin_diag, r->forcing, r->part, r->err,  r->k2_scratch, r->k3g_scratch, r->k3p_scratch,
                   r->k3t_factors, r->k3t_scratch, r->k3d_factors, r->k3d_scratch, r->k3o_factors, r->k3o_scratch,
                   r->k1p_dg, r->k1p_tg, r->probe, r->svd_ut, r->svd_sigma, r->svd_beta, r->k1pp_scratch,
-                  r->k2_tiles};
+                  r->k2_tiles, r->k1t_scratch, r->k1t.d_off, r->k1t.d_ranges};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (cudaEvent_t e : r->prof_ev) cudaEventDestroy(e);
@@ -456,6 +458,21 @@ static cudaError_t svd_beta(grom_rom* r, int batch, const double* u, int64_t u_s
                             active, r->svd_beta, s);
 }
 
+// Arguments of the folded skew-packed kernels for a trajectory batch (ring
+// addressing) or plain buffers, which the caller sets.
+static K1TArgs k1t_args(const grom_rom* r, const grom_traj* t) {
+  K1TArgs a{};
+  a.tensor = r->op;
+  a.err = r->err;
+  if (t) {
+    a.hist = t->hist;
+    a.taken = t->taken;
+    a.hist_stride = 6 * (int64_t)r->n;
+    a.active = t->active;
+  }
+  return a;
+}
+
 static K3Args k3_args(grom_rom* r) {
   K3Args a{};
   a.fa = r->op;
@@ -558,17 +575,36 @@ grom_status grom_create(const grom_desc* d, void* stream, grom_rom** out) {
     const bool packed = r->layout == GROM_LAYOUT_SKEW_PACKED;
     r->k1 = k1_plan(n, r->storage, r->sm_count, packed ? 1 : 0);
     const size_t row_bytes = (size_t)r->k1.row_bytes;
-    r->op_bytes = (size_t)n * (size_t)n * row_bytes;
+    r->folded = packed && (r->storage == GROM_F64 || r->storage == GROM_F32X2);
+    if (r->folded) r->k1t = k1t_plan(n, r->storage, r->sm_count);
+    r->op_bytes = r->folded ? r->k1t.bytes : (size_t)n * (size_t)n * row_bytes;
     if ((st = dmalloc(&r->op, r->op_bytes, &r->total_bytes))) return bail(st);
-    r->part_bytes = (size_t)r->k1.grid * r->k1.maxseg * (K1_CONSUMERS / 32) * r->k1.nb_max * sizeof(double);
-    if ((st = dmalloc(&r->part, r->part_bytes, &r->total_bytes))) return bail(st);
+    if (!r->folded) {
+      r->part_bytes = (size_t)r->k1.grid * r->k1.maxseg * (K1_CONSUMERS / 32) * r->k1.nb_max * sizeof(double);
+      if ((st = dmalloc(&r->part, r->part_bytes, &r->total_bytes))) return bail(st);
+    }
     if (packed) {
+      if ((st = dmalloc(&r->probe, 3 * sizeof(double), &r->total_bytes))) return bail(st);
+      if (cudaMemsetAsync(r->probe, 0, 3 * sizeof(double), r->stream) != cudaSuccess)
+        return bail(cuda_fail(cudaGetLastError(), "grom_create"));
+    }
+    if (r->folded) {
+      const K1TPlan& p = r->k1t;
+      const size_t ob = p.off.size() * sizeof(int64_t), rb = p.ranges.size() * sizeof(int4);
+      if ((st = dmalloc(&r->k1t_scratch, k1t_scratch_bytes(p), &r->total_bytes))) return bail(st);
+      if ((st = dmalloc(&r->k1t.d_off, ob, &r->total_bytes))) return bail(st);
+      if ((st = dmalloc(&r->k1t.d_ranges, rb, &r->total_bytes))) return bail(st);
+      // zeros: the padding of the rows, and the barrier word
+      if (cudaMemsetAsync(r->op, 0, r->op_bytes, r->stream) != cudaSuccess ||
+          cudaMemsetAsync(r->k1t_scratch, 0, 256, r->stream) != cudaSuccess ||
+          cudaMemcpyAsync(p.d_off, p.off.data(), ob, cudaMemcpyHostToDevice, r->stream) != cudaSuccess ||
+          cudaMemcpyAsync(p.d_ranges, p.ranges.data(), rb, cudaMemcpyHostToDevice, r->stream) != cudaSuccess)
+        return bail(cuda_fail(cudaGetLastError(), "grom_create"));
+    } else if (packed) {
       if ((st = dmalloc(&r->k1p_dg, k1p_dg_bytes(r->k1, r->storage), &r->total_bytes))) return bail(st);
       if ((st = dmalloc(&r->k1p_tg, k1p_tg_bytes(r->k1), &r->total_bytes))) return bail(st);
-      if ((st = dmalloc(&r->probe, 3 * sizeof(double), &r->total_bytes))) return bail(st);
       if ((st = dmalloc(&r->k1pp_scratch, k1pp_scratch_bytes(r->k1), &r->total_bytes))) return bail(st);
-      if (cudaMemsetAsync(r->probe, 0, 3 * sizeof(double), r->stream) != cudaSuccess ||
-          cudaMemsetAsync(r->k1pp_scratch, 0, k1pp_scratch_bytes(r->k1), r->stream) != cudaSuccess)
+      if (cudaMemsetAsync(r->k1pp_scratch, 0, k1pp_scratch_bytes(r->k1), r->stream) != cudaSuccess)
         return bail(cuda_fail(cudaGetLastError(), "grom_create"));
     }
     if (r->storage == GROM_BF16 && packed) {
@@ -904,6 +940,15 @@ grom_status grom_nonlinear(grom_rom* r, int32_t batch, const double* u, double* 
     a.err = r->err;
     if (!prof_pair(r, &a.ev0, &a.ev1)) return fail(GROM_ERR_CUDA, "event creation failed");
     e = k2p_launch(k2p_plan_of(r, batch), &r->k2_tmap, a, r->stream);
+  } else if (r->folded) {
+    K1TArgs a = k1t_args(r, nullptr);
+    a.u = u;
+    a.u_stride = r->n;
+    a.c = c;
+    a.c_stride = r->n;
+    cudaEvent_t e0, e1;
+    if (!prof_pair(r, &e0, &e1)) return fail(GROM_ERR_CUDA, "event creation failed");
+    e = k1t_launch(r->k1t, a, batch, r->k1t_scratch, e0, e1, r->stream);
   } else if (!is_cp(r)) {
     K1Args a = k1_args(r);
     a.u = u;
@@ -1034,6 +1079,11 @@ static cudaError_t traj_nonlinear(grom_traj* t, cudaStream_t strm) {
     if (!prof_pair(r, &a.ev0, &a.ev1)) return cudaErrorMemoryAllocation;
     return k2p_launch(k2p_plan_of(r, t->batch), &r->k2_tmap, a, strm);
   }
+  if (r->folded) {
+    cudaEvent_t e0, e1;
+    if (!prof_pair(r, &e0, &e1)) return cudaErrorMemoryAllocation;
+    return k1t_launch(r->k1t, k1t_args(r, t), t->batch, r->k1t_scratch, e0, e1, strm);
+  }
   if (!is_cp(r)) {
     K1Args a = k1_args(r);
     a.hist = t->hist;
@@ -1117,7 +1167,7 @@ static StepArgs step_args(grom_traj* t, double* energy, double* invariant) {
 static cudaError_t launch_steps(grom_traj* t, int count, double* energy, double* invariant, cudaStream_t strm) {
   grom_rom* r = t->rom;
   StepArgs a = step_args(t, energy, invariant);
-  const bool fused_k1 = r->diagonal && !is_cp(r) && !use_k2(r, t->batch) && !use_k2p(r, t->batch);
+  const bool fused_k1 = r->diagonal && !is_cp(r) && !r->folded && !use_k2(r, t->batch) && !use_k2p(r, t->batch);
   const bool fused_k3 = r->diagonal && is_cp(r) && !use_k3g(r, t->batch) && !use_k3t(r, t->batch);
   const bool fused_k3t = r->diagonal && use_k3t(r, t->batch);
   const bool fused_k3d = r->diagonal && use_k3d(r, t->batch) && !use_k3o(r, t->batch);
@@ -1198,9 +1248,24 @@ static cudaError_t launch_steps(grom_traj* t, int count, double* energy, double*
 // launch.
 static bool persistent_ok(const grom_traj* t, int nsteps) {
   const grom_rom* r = t->rom;
-  return r->form == GROM_FORM_FULL && r->layout == GROM_LAYOUT_SKEW_PACKED && r->diagonal && r->k1pp_scratch &&
-         !t->active && t->batch <= 4 && t->batch <= r->k1.nb_max && nsteps >= 1 &&
+  return r->form == GROM_FORM_FULL && r->layout == GROM_LAYOUT_SKEW_PACKED && r->diagonal && !t->active &&
+         t->batch <= 4 && t->batch <= (r->folded ? r->k1t.nb_max : r->k1.nb_max) && nsteps >= 1 &&
          r->kernel_choice != GROM_KERNEL_STREAM && !use_k2p(r, t->batch, false);
+}
+
+// The whole call on the persistent stepper of the ROM's layout.
+static cudaError_t launch_persistent(grom_traj* t, int nsteps, double* energy, double* invariant, cudaEvent_t e0,
+                                     cudaEvent_t e1, cudaStream_t strm) {
+  grom_rom* r = t->rom;
+  const StepArgs a = step_args(t, energy, invariant);
+  if (r->folded) return k1tp_launch(r->k1t, k1t_args(r, t), a, t->batch, nsteps, r->k1t_scratch, e0, e1, strm);
+  K1Args k = k1_args(r);
+  k.hist = t->hist;
+  k.taken = t->taken;
+  k.hist_stride = 6 * (int64_t)r->n;
+  k.ev0 = e0;
+  k.ev1 = e1;
+  return k1pp_launch(r->k1, r->storage, k, a, t->batch, nsteps, r->k1pp_scratch, strm);
 }
 
 grom_status grom_step(grom_traj* t, int32_t nsteps, double* energy, double* invariant) {
@@ -1223,16 +1288,9 @@ grom_status grom_step(grom_traj* t, int32_t nsteps, double* energy, double* inva
   // in one persistent launch (falls back to the graphs below when the launch
   // cannot be placed)
   if (persistent_ok(t, nsteps)) {
-    StepArgs a = step_args(t, energy, invariant);
-    K1Args k = k1_args(r);
-    k.hist = t->hist;
-    k.taken = t->taken;
-    k.hist_stride = 6 * (int64_t)r->n;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!prof_pair(r, &e0, &e1)) return fail(GROM_ERR_CUDA, "event creation failed");
-    k.ev0 = e0;
-    k.ev1 = e1;
-    const cudaError_t e = k1pp_launch(r->k1, r->storage, k, a, t->batch, nsteps, r->k1pp_scratch, r->stream);
+    const cudaError_t e = launch_persistent(t, nsteps, energy, invariant, e0, e1, r->stream);
     if (e == cudaSuccess) return GROM_OK;
     if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorInvalidValue)
       return cuda_fail(e, "grom_step persistent launch");
@@ -1415,12 +1473,7 @@ grom_status grom_step_host(grom_traj* t, int32_t nsteps, const double* u_in, dou
         }
         if (e == cudaSuccess) {
           if (persist) {
-            StepArgs a = step_args(t, nullptr, nullptr);
-            K1Args k = k1_args(r);
-            k.hist = t->hist;
-            k.taken = t->taken;
-            k.hist_stride = 6 * (int64_t)r->n;
-            e = k1pp_launch(r->k1, r->storage, k, a, t->batch, nsteps, r->k1pp_scratch, t->gstream);
+            e = launch_persistent(t, nsteps, nullptr, nullptr, nullptr, nullptr, t->gstream);
           } else {
             e = launch_steps(t, nsteps, nullptr, nullptr, t->gstream);
           }

@@ -35,6 +35,61 @@ __device__ __forceinline__ void ds_mac(float ah, float al, float bh, float bl, f
   S = S1;
 }
 
+// Two independent FP32 values in a register pair (low word first) and the
+// packed operations on them: each rounds as its scalar counterpart, in one
+// issue slot for both.
+struct f32pair {
+  unsigned long long v;
+};
+__device__ __forceinline__ f32pair pair_make(float x, float y) {
+  f32pair r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void pair_get(f32pair a, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v));
+}
+__device__ __forceinline__ f32pair pair_add(f32pair a, f32pair b) {
+  f32pair r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+// The product as two scalar instructions: the assembler contracts a packed
+// multiplication with the addition that uses it, .rn or not, and a fused
+// first sum breaks the transformation below (5e-9 instead of 1e-14 a sum).
+__device__ __forceinline__ f32pair pair_mul(f32pair a, f32pair b) {
+  float a0, a1, b0, b1;
+  pair_get(a, a0, a1);
+  pair_get(b, b0, b1);
+  return pair_make(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
+}
+__device__ __forceinline__ f32pair pair_fma(f32pair a, f32pair b, f32pair c) {
+  f32pair r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ f32pair pair_sub(f32pair a, f32pair b) {  // a - b
+  return pair_fma(b, f32pair{0xBF800000BF800000ull}, a);
+}
+
+// ds_mac for two accumulators: the same operations and roundings (-bb formed
+// as S - S1), eleven issue slots for the two.
+__device__ __forceinline__ void ds_mac2(f32pair ah, f32pair al, f32pair bh, f32pair bl, f32pair& S, f32pair& s) {
+  const f32pair S1 = pair_add(S, pair_mul(ah, bh));
+  const f32pair nb = pair_sub(S, S1);
+  const f32pair y = pair_sub(S, pair_add(S1, nb));
+  f32pair w = pair_add(y, pair_fma(ah, bh, nb));
+  w = pair_fma(al, bh, w);
+  w = pair_fma(ah, bl, w);
+  s = pair_add(s, w);
+  S = S1;
+}
+__device__ __forceinline__ void ds_renorm2(f32pair& S, f32pair& s) {
+  const f32pair h = pair_add(S, s);
+  s = pair_sub(s, pair_sub(h, S));
+  S = h;
+}
+
 // Fast2Sum: the pair as its rounded sum and that sum's error.
 __device__ __forceinline__ void ds_renorm(float& S, float& s) {
   const float h = __fadd_rn(S, s);

@@ -60,6 +60,7 @@ inline int storage_elem_bytes(int storage) {
 }  // namespace grom
 
 #include "k1_types.h"
+#include "k1t_types.h"
 
 namespace grom {
 
@@ -387,6 +388,10 @@ cudaError_t step_diag_mc_k3t_launch(const StepArgs& a, int step_index, const K3T
 cudaError_t step_diag_mc_k3d_launch(const StepArgs& a, int step_index, const K3TStepFuse& f, cudaStream_t s);
 cudaError_t step_diag_packed_launch(const StepArgs& a, int step_index, const K1Plan& pl, const K1Args& k1a, int b0,
                                     int nb, int nbk, cudaStream_t s);
+// Persistent stepper of the folded skew-packed layout (k1t.cuh): nsteps
+// diagonal steps of up to nb_max trajectories in one cooperative launch.
+cudaError_t k1tp_launch(const K1TPlan& p, K1TArgs a, const StepArgs& st, int batch, int nsteps, void* scratch,
+                        cudaEvent_t ev0, cudaEvent_t ev1, cudaStream_t s);
 // Persistent skew-packed stepper (k1p_persist.cuh): nsteps diagonal steps of
 // up to 4 trajectories in one cooperative launch.  scratch: k1pp_scratch_bytes,
 // zeroed once at creation.  Returns an error without launching when the plan
@@ -460,6 +465,9 @@ struct grom_rom {
   double* svd_sigma = nullptr;  // SVD form: singular values (rank)
   double* svd_beta = nullptr;   // SVD form: middle weights (max_batch x rank)
   grom::K1Plan k1{};
+  bool folded = false;          // skew-packed F64 / F32X2 full form: the folded layout (k1t)
+  grom::K1TPlan k1t;
+  void* k1t_scratch = nullptr;  // its barrier word, partials and windows
   grom::K3Plan k3{};
   size_t total_bytes = 0;
   int traj_count = 0;

@@ -12,8 +12,6 @@ cudaError_t k1p_dispatch_f64(int qm, int nb, const K1Plan&, const K1Args&, int, 
 cudaError_t k1p_dispatch_f32x2(int qm, int nb, const K1Plan&, const K1Args&, int, cudaStream_t);
 cudaError_t k1p_dispatch_f32(int qm, int nb, const K1Plan&, const K1Args&, int, cudaStream_t);
 cudaError_t k1p_dispatch_bf16(int qm, int nb, const K1Plan&, const K1Args&, int, cudaStream_t);
-cudaError_t k1pp_dispatch_f64(int, int, const K1Plan&, const K1Args&, const StepArgs&, const K1PPArgs&, cudaStream_t);
-cudaError_t k1pp_dispatch_f32x2(int, int, const K1Plan&, const K1Args&, const StepArgs&, const K1PPArgs&, cudaStream_t);
 cudaError_t k1pp_dispatch_f32(int, int, const K1Plan&, const K1Args&, const StepArgs&, const K1PPArgs&, cudaStream_t);
 cudaError_t k1pp_dispatch_bf16(int, int, const K1Plan&, const K1Args&, const StepArgs&, const K1PPArgs&, cudaStream_t);
 
@@ -196,8 +194,6 @@ cudaError_t k1pp_launch(const K1Plan& plan, int storage, const K1Args& a0, const
   pp.red = reinterpret_cast<double*>(reinterpret_cast<uint8_t*>(scratch) + 256);
   pp.nsteps = nsteps;
   switch (storage) {
-    case GROM_F64: return k1pp_dispatch_f64(pl.qm, nb, pl, a, st, pp, s);
-    case GROM_F32X2: return k1pp_dispatch_f32x2(pl.qm, nb, pl, a, st, pp, s);
     case GROM_F32: return k1pp_dispatch_f32(pl.qm, nb, pl, a, st, pp, s);
     case GROM_BF16: return k1pp_dispatch_bf16(pl.qm, nb, pl, a, st, pp, s);
   }

@@ -1,4 +1,5 @@
-// Persistent stepper of the G-ROM with the skew-packed tensor: many
+// Persistent stepper of the G-ROM with the skew-packed FP32 or BF16 tensor (FP64
+// and F32X2: k1t.cuh): many
 // BDFk/EXTk steps (Sec. 2.2, eq. nse_d1) in one cooperative launch.
 //
 // Every CTA keeps the stage ring of the packed streaming kernel
@@ -138,17 +139,11 @@ __global__ void __launch_bounds__(K1_THREADS, 1)
     const int64_t uplane = (int64_t)NB * np;
     const int64_t first_i = c0 / pl.cpi, last_i = (c1 - 1) / pl.cpi;
     const int64_t nseg = last_i - first_i + 1;
-    constexpr int RMAX = k1_rmax(QM, (ST == GROM_F32X2) ? 2 : 1);
-    constexpr int PLANES = (ST == GROM_F32X2) ? 2 : 1;
+    constexpr int RMAX = k1_rmax(QM, 1);
     const int t_off = (int)(ro * row_bytes + pos0 * 16);
     const int t_step = (int)(R * row_bytes);
     const int q_step = W * 16;
-    const int plane_off = (int)(lp * 4);
     const bool full_pos = act && (pos0 + (QM - 1) * W < P);
-    // rows of a full chunk held by this thread (other chunks: the last of a test index)
-    int nrow_full = act ? ((int)pl.rpc - ro + R - 1) >> lgR : 0;
-    if (nrow_full > RMAX) nrow_full = RMAX;
-    if (nrow_full < 0) nrow_full = 0;
     const int64_t i_lo = (int64_t)g * n / G, i_hi = ((int64_t)g + 1) * n / G;  // owned test indices
     int s = 0;
     uint32_t ph = 0;
@@ -161,15 +156,7 @@ __global__ void __launch_bounds__(K1_THREADS, 1)
         const int64_t k = idx - (int64_t)b * np;
         double v = 0.0;
         if (b < nb && k < n) v = __ldcg(a.hist + b * a.hist_stride + ((l0s[b] + step) % 3) * n + k);
-        if constexpr (ST == GROM_F64) {
-          reinterpret_cast<double*>(ureg)[idx] = v;
-        } else if constexpr (ST == GROM_F32X2) {
-          const float hv = __double2float_rn(v);
-          reinterpret_cast<float*>(ureg)[idx] = hv;
-          reinterpret_cast<float*>(ureg)[uplane + idx] = __double2float_rn(v - (double)hv);
-        } else {
-          reinterpret_cast<float*>(ureg)[idx] = __double2float_rn(v);
-        }
+        reinterpret_cast<float*>(ureg)[idx] = __double2float_rn(v);
       }
       ptx::named_sync(1, K1_CONSUMERS);
 
@@ -197,23 +184,10 @@ __global__ void __launch_bounds__(K1_THREADS, 1)
           for (int e = 0; e < TR::EPV; ++e) {
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
-              double v;
-              if constexpr (ST == GROM_BF16 || ST == GROM_F32) {
-                float f = acc[q][e][b].v;
-                if (R >= 2) f += __shfl_xor_sync(0xffffffffu, f, 8);
-                if (R >= 4) f += __shfl_xor_sync(0xffffffffu, f, 16);
-                v = (double)f;
-              } else {
-                double d;
-                if constexpr (ST == GROM_F64) {
-                  d = acc[q][e][b].v;
-                } else {
-                  d = (double)acc[q][e][b].S + (double)acc[q][e][b].s;
-                }
-                if (R >= 2) d += __shfl_xor_sync(0xffffffffu, d, 8);
-                if (R >= 4) d += __shfl_xor_sync(0xffffffffu, d, 16);
-                v = d;
-              }
+              float f = acc[q][e][b].v;
+              if (R >= 2) f += __shfl_xor_sync(0xffffffffu, f, 8);
+              if (R >= 4) f += __shfl_xor_sync(0xffffffffu, f, 16);
+              const double v = (double)f;
               acc[q][e][b].zero();
               if (ro == 0 && pos < P) {
                 const int64_t p = (int64_t)pos * TR::EPV + e;
@@ -265,91 +239,41 @@ __global__ void __launch_bounds__(K1_THREADS, 1)
           break;
         }
         const uint8_t* stg = stages + s * K1_STAGE_BYTES + t_off;
-        int nrow;
-        if constexpr (ST == GROM_F32X2) {
-          // full chunks: the precomputed count
-          nrow = nrow_full;
-          if (rows != (int)pl.rpc) {
-            nrow = act ? (rows - ro + R - 1) >> lgR : 0;
-            if (nrow > RMAX) nrow = RMAX;
-            if (nrow < 0) nrow = 0;
-          }
-        } else {
-          // (the precomputed count measured 6 % slower here for BF16 on GB300)
-          nrow = act ? (rows - ro + R - 1) / R : 0;
-          if (nrow > RMAX) nrow = RMAX;
-          if (nrow < 0) nrow = 0;
-        }
-        uint4 vec[RMAX][QM][PLANES];
+        // (a count formed before the loop measured 6 % slower here for BF16 on GB300)
+        int nrow = act ? (rows - ro + R - 1) / R : 0;
+        if (nrow > RMAX) nrow = RMAX;
+        if (nrow < 0) nrow = 0;
+        uint4 vec[RMAX][QM];
         if (full_pos && nrow == RMAX) {
 #pragma unroll
           for (int t = 0; t < RMAX; ++t)
 #pragma unroll
             for (int q = 0; q < QM; ++q)
-#pragma unroll
-              for (int p2 = 0; p2 < PLANES; ++p2)
-                vec[t][q][p2] = *reinterpret_cast<const uint4*>(stg + t * t_step + q * q_step + p2 * plane_off);
+              vec[t][q] = *reinterpret_cast<const uint4*>(stg + t * t_step + q * q_step);
         } else {
 #pragma unroll
           for (int t = 0; t < RMAX; ++t)
 #pragma unroll
             for (int q = 0; q < QM; ++q) {
               const bool ok = t < nrow && (pos0 + q * W < P);
-#pragma unroll
-              for (int p2 = 0; p2 < PLANES; ++p2)
-                vec[t][q][p2] = ok ? *reinterpret_cast<const uint4*>(stg + t * t_step + q * q_step + p2 * plane_off)
-                                   : make_uint4(0, 0, 0, 0);
+              vec[t][q] = ok ? *reinterpret_cast<const uint4*>(stg + t * t_step + q * q_step) : make_uint4(0, 0, 0, 0);
             }
         }
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&empty[s]);
         if (++s == K1_STAGES) { s = 0; ph ^= 1u; }
         const int jt = j0 + ro;
-        ds_renorm_all<ST>(acc);
 #pragma unroll
         for (int t = 0; t < RMAX; ++t) {
           if (t >= nrow) break;
           const int j = jt + t * R;
-          if constexpr (ST == GROM_F64) {
-            double uj[NB];
-#pragma unroll
-            for (int b = 0; b < NB; ++b) uj[b] = reinterpret_cast<const double*>(ureg)[b * (int)np + j];
-#pragma unroll
-            for (int q = 0; q < QM; ++q) {
-              const double x0 = __hiloint2double((int)vec[t][q][0].y, (int)vec[t][q][0].x);
-              const double x1 = __hiloint2double((int)vec[t][q][0].w, (int)vec[t][q][0].z);
-#pragma unroll
-              for (int b = 0; b < NB; ++b) {
-                acc[q][0][b].v = fma(x0, uj[b], acc[q][0][b].v);
-                acc[q][1][b].v = fma(x1, uj[b], acc[q][1][b].v);
-              }
-            }
-          } else if constexpr (ST == GROM_F32X2) {
-            float uh[NB], ul[NB];
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-              uh[b] = reinterpret_cast<const float*>(ureg)[b * (int)np + j];
-              ul[b] = reinterpret_cast<const float*>(ureg)[(NB + b) * (int)np + j];
-            }
-#pragma unroll
-            for (int q = 0; q < QM; ++q) {
-              const uint4 hv = vec[t][q][0];
-              const uint4 lv = vec[t][q][PLANES - 1];
-#pragma unroll
-              for (int b = 0; b < NB; ++b) {
-                ds_mac(__uint_as_float(hv.x), __uint_as_float(lv.x), uh[b], ul[b], acc[q][0][b].S, acc[q][0][b].s);
-                ds_mac(__uint_as_float(hv.y), __uint_as_float(lv.y), uh[b], ul[b], acc[q][1][b].S, acc[q][1][b].s);
-                ds_mac(__uint_as_float(hv.z), __uint_as_float(lv.z), uh[b], ul[b], acc[q][2][b].S, acc[q][2][b].s);
-                ds_mac(__uint_as_float(hv.w), __uint_as_float(lv.w), uh[b], ul[b], acc[q][3][b].S, acc[q][3][b].s);
-              }
-            }
-          } else if constexpr (ST == GROM_F32) {
+          if constexpr (ST == GROM_F32) {
             float uj[NB];
 #pragma unroll
             for (int b = 0; b < NB; ++b) uj[b] = reinterpret_cast<const float*>(ureg)[b * (int)np + j];
 #pragma unroll
             for (int q = 0; q < QM; ++q) {
-              const uint4 x = vec[t][q][0];
+              const uint4 x = vec[t][q];
 #pragma unroll
               for (int b = 0; b < NB; ++b) {
                 acc[q][0][b].v = fmaf(__uint_as_float(x.x), uj[b], acc[q][0][b].v);
@@ -364,7 +288,7 @@ __global__ void __launch_bounds__(K1_THREADS, 1)
             for (int b = 0; b < NB; ++b) uj[b] = reinterpret_cast<const float*>(ureg)[b * (int)np + j];
 #pragma unroll
             for (int q = 0; q < QM; ++q) {
-              const uint32_t ws[4] = {vec[t][q][0].x, vec[t][q][0].y, vec[t][q][0].z, vec[t][q][0].w};
+              const uint32_t ws[4] = {vec[t][q].x, vec[t][q].y, vec[t][q].z, vec[t][q].w};
 #pragma unroll
               for (int hh = 0; hh < 4; ++hh) {
                 const float x0 = __uint_as_float(ws[hh] << 16);

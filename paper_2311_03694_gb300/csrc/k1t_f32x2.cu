@@ -1,0 +1,16 @@
+// Folded skew-packed streaming kernel, GROM_F32X2 storage.
+#include "k1t.cuh"
+
+namespace grom {
+
+cudaError_t k1t_dispatch_f32x2(int qm, int nb, const K1TArgs& a, const StepArgs& st, int grid, size_t smem,
+                               cudaStream_t s) {
+  switch (qm) {
+    case 1: return k1t_pick_nb<GROM_F32X2, 1>(nb, a, st, grid, smem, s);
+    case 2: return k1t_pick_nb<GROM_F32X2, 2>(nb, a, st, grid, smem, s);
+    case 4: return k1t_pick_nb<GROM_F32X2, 4>(nb, a, st, grid, smem, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace grom

@@ -346,7 +346,7 @@ __global__ void k2_prep_kernel(const K2Dev p, const double* u, int64_t u_stride,
 // time.  What bounds it is reading the partials once.  Summing them in FP64
 // was bound by that pipe instead (a conversion and an addition per partial
 // at two a clock and SM: n = 512, 256 trajectories, 76 splits, 47 us); the
-// triple-float sums keep more bits and take 17.5 us  A sum that leaves
+// triple-float sums keep more bits and take 17.5 us.  A sum that leaves
 // the FP32 range (or holds an infinity or a NaN) is done again in FP64.
 constexpr int K2R_I = 16, K2R_B = 32;
 __global__ void __launch_bounds__(K2R_I * K2R_B / 4)
