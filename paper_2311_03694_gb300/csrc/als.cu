@@ -17,12 +17,12 @@
 // rank^3/3 + 2 n rank^2 flops per update).  Only the Cholesky breakdown flag,
 // the residual's two sums and the final factors come back to the host.
 #include <algorithm>
-#include <chrono>
 #include <cmath>
 #include <cstring>
 #include <new>
 #include <vector>
 
+#include "ds_arith.cuh"
 #include "grom_internal.h"
 
 using namespace grom;
@@ -51,9 +51,12 @@ struct grom_als {
   int* flag = nullptr;                            // Cholesky breakdown
   void* k2s = nullptr;
   size_t k2s_bytes = 0;
-  // timing since the last grom_als_stats: MTTKRP device time (CUDA events
-  // around each tensor-core launch) and wall time of the SPD solves
+  // timing since the last grom_als_stats: device times (CUDA events) of the
+  // tensor-core launches and of the SPD solves (the part of a factorisation
+  // that outlasts its MTTKRP, and the triangular solves)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  cudaStream_t side = nullptr;                    // the factorisations' stream
+  cudaEvent_t fork = nullptr, join = nullptr, sv0 = nullptr, sv1 = nullptr;
   double mttkrp_ms = 0.0, solve_ms = 0.0;
   int64_t mttkrp_calls = 0;
 };
@@ -114,22 +117,41 @@ __global__ void k_als_norm(const double* __restrict__ src, int64_t total, double
 
 // G = F^T F for F (n x r, row-major FP64), 16 x 16 output tiles; G is
 // symmetric, so only the tiles on and above the diagonal are computed (FP64
-// runs at about two operations per clock per SM here) and mirrored.
-__global__ void k_gram(const double* __restrict__ F, int64_t n, int64_t r, double* __restrict__ G) {
+// runs at about two operations per clock per SM here) and mirrored.  Chunks
+// of 64 rows with the next one in flight, so that two warps per FP64 pipe
+// keep it busy (n = 512, r = 256: 68.4 us against 75.8 with chunks of
+// 16; the pipe's own time is 32 us).
+constexpr int GR_K = 64;
+__global__ void __launch_bounds__(256) k_gram(const double* __restrict__ F, int64_t n, int64_t r,
+                                              double* __restrict__ G) {
   if (blockIdx.x < blockIdx.y) return;  // whole block, before any barrier
-  __shared__ double a[16][17], b[16][17];
+  __shared__ double a[GR_K][17], b[GR_K][17];
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int64_t row = (int64_t)blockIdx.y * 16 + ty, col = (int64_t)blockIdx.x * 16 + tx;
-  double s = 0.0;
-  for (int64_t i0 = 0; i0 < n; i0 += 16) {
-    const int64_t i = i0 + ty;
-    a[ty][tx] = (i < n && (int64_t)blockIdx.y * 16 + tx < r) ? F[i * r + blockIdx.y * 16 + tx] : 0.0;
-    b[ty][tx] = (i < n && col < r) ? F[i * r + col] : 0.0;
-    __syncthreads();
+  const int64_t ra = (int64_t)blockIdx.y * 16 + tx, col = (int64_t)blockIdx.x * 16 + tx;
+  double na[GR_K / 16], nb[GR_K / 16];
+  auto fetch = [&](int64_t i0) {
 #pragma unroll
-    for (int q = 0; q < 16; ++q) s = fma(a[q][ty], b[q][tx], s);
+    for (int k = 0; k < GR_K / 16; ++k) {
+      const int64_t i = i0 + 16 * k + ty;
+      na[k] = i < n && ra < r ? F[i * r + ra] : 0.0;
+      nb[k] = i < n && col < r ? F[i * r + col] : 0.0;
+    }
+  };
+  fetch(0);
+  double s = 0.0;
+  for (int64_t i0 = 0; i0 < n; i0 += GR_K) {
+#pragma unroll
+    for (int k = 0; k < GR_K / 16; ++k) {
+      a[16 * k + ty][tx] = na[k];
+      b[16 * k + ty][tx] = nb[k];
+    }
+    __syncthreads();
+    if (i0 + GR_K < n) fetch(i0 + GR_K);
+#pragma unroll 16
+    for (int q = 0; q < GR_K; ++q) s = fma(a[q][ty], b[q][tx], s);
     __syncthreads();
   }
+  const int64_t row = (int64_t)blockIdx.y * 16 + ty;
   if (row < r && col < r) {
     G[row * r + col] = s;
     G[col * r + row] = s;
@@ -175,42 +197,49 @@ __device__ __forceinline__ double rsqrt_nr(double d) {
   return scalbn(y, -e);
 }
 
-// Factors the diagonal block at (kb, kb) in place (lower), one thread per
-// entry (32 x 32), right-looking, and stores the reciprocals of its pivots
-// in rdiag[kb ..].  A pivot that is not positive and finite sets *flag.
-__global__ void __launch_bounds__(CH * CH) k_chol_diag(double* H, int64_t r, int64_t kb, double* rdiag, int* flag) {
-  __shared__ double A[CH][CH + 1];
-  __shared__ double ry;
-  __shared__ int bad;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // entry A[ty][tx]
+// Factors the diagonal block at (kb, kb) in place (lower), right-looking, and
+// stores the reciprocals of its pivots in rdiag[kb ..].  A pivot that is not
+// positive and finite sets *flag.  One CTA of four warps, one per FP64 pipe:
+// lane = column, warp w holds rows w, w + 4, ... in registers, every warp
+// forms the pivot's reciprocal root itself, and the next column goes through
+// shared memory: one barrier a pivot, where a thread per entry took three.
+// The chain of some ten dependent FP64 operations a pivot is what bounds it:
+// 38.2 us a block against 50.5.
+__global__ void __launch_bounds__(128) k_chol_diag(double* H, int64_t r, int64_t kb, double* rdiag, int* flag) {
+  __shared__ double Ls[CH][CH + 1], col[2][CH];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nb = (int)(r - kb < CH ? r - kb : CH);
-  if (ty < nb && tx < nb) A[ty][tx] = H[(kb + ty) * r + kb + tx];
-  if (threadIdx.x == 0) bad = 0;
+  double a[CH / 4];
+#pragma unroll
+  for (int k = 0; k < CH / 4; ++k) {
+    const int i = w + 4 * k;
+    a[k] = i < nb && lane <= i ? H[(kb + i) * r + kb + lane] : (lane == i ? 1.0 : 0.0);
+    if (lane == 0) col[0][i] = a[k];
+  }
   __syncthreads();
   for (int c = 0; c < nb; ++c) {
-    if (threadIdx.x == 0) {
-      const double d = A[c][c];
-      if (!(d > 0.0) || !isfinite(d)) {
-        bad = 1;
-      } else {
-        const double y = rsqrt_nr(d);
-        A[c][c] = d * y;
-        ry = y;
-        rdiag[kb + c] = y;
-      }
+    const double* cc = col[c & 1];  // column c, rows >= c
+    const double d = cc[c];
+    if (!(d > 0.0) || !isfinite(d)) {  // the same value in every thread
+      if (threadIdx.x == 0) atomicExch(flag, 1);
+      return;
+    }
+    const double y = rsqrt_nr(d);
+    const double l = cc[lane] * y;  // L[lane][c] for lane > c
+    if (w == 0) Ls[lane][c] = lane > c ? l : lane == c ? d * y : 0.0;
+    if (w == 1 && lane == 0) rdiag[kb + c] = y;
+#pragma unroll
+    for (int k = 0; k < CH / 4; ++k) {
+      const int i = w + 4 * k;
+      const double li = __shfl_sync(0xffffffffu, l, i);
+      if (i <= c) continue;  // warp-uniform
+      a[k] = fma(-li, l, a[k]);
+      if (lane == c + 1) col[(c + 1) & 1][i] = a[k];
     }
     __syncthreads();
-    if (bad) break;  // read by every thread between the same two barriers
-    if (tx == c && ty > c && ty < nb) A[ty][c] *= ry;
-    __syncthreads();
-    if (ty > c && ty < nb && tx > c && tx <= ty) A[ty][tx] -= A[ty][c] * A[tx][c];
-    __syncthreads();
   }
-  if (bad) {
-    if (threadIdx.x == 0) atomicExch(flag, 1);
-    return;
-  }
-  if (ty < nb && tx < nb) H[(kb + ty) * r + kb + tx] = tx <= ty ? A[ty][tx] : 0.0;
+  for (int x = threadIdx.x; x < nb * CH; x += 128)
+    if (x % CH < nb) H[(kb + x / CH) * r + kb + x % CH] = Ls[x / CH][x % CH];
 }
 
 // Rows i >= kb + CH: H[i][kb .. kb+CH) <- H[i][kb .. kb+CH) L11^-T (one warp
@@ -265,96 +294,96 @@ __global__ void k_transpose(const double* __restrict__ L, int64_t r, double* __r
   }
 }
 
-// Lane t of the warp ends with the sum over the 32 lanes of v[t].
-__device__ __forceinline__ double warp_transpose_sum(double (&v)[32], int lane) {
+// A[i][:] = M[i][:] H^-1 (M given transposed, r x n; H = L L^T): forward
+// L z = m_i, backward L^T a_i = z, 32 unknowns at a time, SV_ROWS rows per CTA
+// and four warps per row.  Per block the solved unknowns' contribution is
+// summed with lanes over the contracted index (coalesced rows of L or L^T,
+// eight unknowns a warp, a butterfly across the lanes), then the row's first
+// warp (the rows of a CTA run at their own pace) solves the 32 x 32 triangle, staged in shared memory with the
+// reciprocals of its pivots, with shuffles.
+// n r^2 multiply-adds (53 us of the FP64 pipe at n = 512, r = 256) and the
+// triangles' chains of 2 r shuffle-multiply-add steps bound it: 221 us
+// there; one warp per row, with 32 sums of its own, took 400.
+constexpr int SV_ROWS = 4, SV_WARPS = 4, SV_T = CH / SV_WARPS;
+
+// Butterfly sums over the 32 lanes of v[0 .. 8): every pair of partial sums
+// is added in the order 16, 8, 4, 2, 1, and lane l ends with v[(l >> 2) & 7]
+// of the order below (bit 4 of the lane picks the upper four, and so on).
+__device__ __forceinline__ double warp_sum8(double (&v)[SV_T], int lane) {
 #pragma unroll
-  for (int s = 16; s >= 1; s >>= 1) {
+  for (int h = SV_T / 2, s = 16; h >= 1; h >>= 1, s >>= 1) {
     const bool up = (lane & s) != 0;
 #pragma unroll
-    for (int c = 0; c < s; ++c) {
-      const double send = up ? v[c] : v[c + s];
-      const double keep = up ? v[c + s] : v[c];
+    for (int c = 0; c < h; ++c) {
+      const double send = up ? v[c] : v[c + h];
+      const double keep = up ? v[c + h] : v[c];
       v[c] = keep + __shfl_xor_sync(0xffffffffu, send, s);
     }
   }
-  return v[0];
+  double x = v[0];
+  x += __shfl_xor_sync(0xffffffffu, x, 2);
+  x += __shfl_xor_sync(0xffffffffu, x, 1);
+  return x;
 }
 
-constexpr int SOLVE_WARPS = 4;
-
-// A[i][:] = M[i][:] H^-1 (M given transposed, r x n; H = L L^T): forward
-// L z = m_i, backward L^T a_i = z, one warp per row i, 32 unknowns at a
-// time.  Per block the earlier unknowns' contribution is summed with lanes
-// over the contracted index (coalesced rows of L or L^T, a transpose-reduce
-// across the lanes), then the 32 x 32 triangle, staged in shared memory with
-// the reciprocals of its pivots, is solved with shuffles.
-
-// The 32 x 32 block of M (row-major, stride r) at (a0, a0) into B (pitch 33)
-// and the reciprocals of its diagonal (rdiag) into column 32; one warp.
-__device__ __forceinline__ void stage_block(const double* __restrict__ M, const double* __restrict__ rdiag, int64_t r,
-                                            int64_t a0, int nb, double (*B)[33], int lane) {
-  for (int t = 0; t < nb; ++t)
-    if (lane < nb) B[t][lane] = M[(a0 + t) * r + a0 + lane];
-  if (lane < nb) B[lane][32] = rdiag[a0 + lane];
-  __syncwarp();
-}
-__global__ void __launch_bounds__(32 * SOLVE_WARPS)
+__global__ void __launch_bounds__(32 * SV_ROWS * SV_WARPS)
     k_als_rowsolve(const double* __restrict__ L, const double* __restrict__ Lt, const double* __restrict__ rdiag,
                    const double* __restrict__ Mt, int64_t n, int64_t r, double* __restrict__ A) {
   extern __shared__ double ybuf[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t i = (int64_t)blockIdx.x * SOLVE_WARPS + w;
-  if (i >= n) return;  // warp-uniform
-  double(*B)[33] = reinterpret_cast<double(*)[33]>(ybuf + (size_t)SOLVE_WARPS * r) + w * 32;
-  double* y = ybuf + (size_t)w * r;
-  for (int64_t c = lane; c < r; c += 32) y[c] = Mt[c * n + i];
-  __syncwarp();
-  for (int64_t a0 = 0; a0 < r; a0 += 32) {
-    const int nb = (int)(r - a0 < 32 ? r - a0 : 32);
-    double acc[32];
-#pragma unroll
-    for (int t = 0; t < 32; ++t) acc[t] = 0.0;
-    for (int64_t q = lane; q < a0; q += 32) {
-      const double yq = y[q];
-#pragma unroll
-      for (int t = 0; t < 32; ++t)
-        if (t < nb) acc[t] = fma(L[(a0 + t) * r + q], yq, acc[t]);
-    }
-    double v = warp_transpose_sum(acc, lane);
-    v = lane < nb ? y[a0 + lane] - v : 0.0;
-    stage_block(L, rdiag, r, a0, nb, B, lane);
-    for (int c = 0; c < nb; ++c) {
-      const double xc = __shfl_sync(0xffffffffu, v, c) * B[c][32];
-      if (lane == c) v = xc;
-      else if (lane > c && lane < nb) v -= B[lane][c] * xc;
-    }
-    if (lane < nb) y[a0 + lane] = v;
-    __syncwarp();
+  __shared__ double Bs[SV_ROWS][CH][CH + 1];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, row = w / SV_WARPS, sub = w % SV_WARPS;
+  const int64_t i0 = (int64_t)blockIdx.x * SV_ROWS, i = i0 + row;
+  const int rt = threadIdx.x % (32 * SV_WARPS);  // thread of the row's four warps
+  double* y = ybuf + (size_t)row * r;
+  double(*B)[CH + 1] = Bs[row];
+  auto row_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(row + 1), "r"(32 * SV_WARPS) : "memory"); };
+  for (int64_t t = threadIdx.x; t < SV_ROWS * r; t += blockDim.x) {
+    const int64_t c = t / SV_ROWS, q = t % SV_ROWS;
+    ybuf[q * r + c] = i0 + q < n ? Mt[c * n + i0 + q] : 0.0;
   }
-  for (int64_t a0 = (r - 1) / 32 * 32; a0 >= 0; a0 -= 32) {
-    const int nb = (int)(r - a0 < 32 ? r - a0 : 32);
-    double acc[32];
+  __syncthreads();
+  const int64_t last = (r - 1) / CH * CH;
+  for (int pass = 0; pass < 2; ++pass) {
+    const double* M = pass ? Lt : L;
+    for (int64_t x = 0; x <= last; x += CH) {
+      const int64_t a0 = pass ? last - x : x;
+      const int nb = (int)(r - a0 < CH ? r - a0 : CH);
+      const int64_t q0 = pass ? a0 + nb : 0, q1 = pass ? r : a0;  // the solved unknowns
+      for (int t = rt; t < CH * CH; t += 32 * SV_WARPS)
+        if (t / CH < nb && t % CH < nb) B[t / CH][t % CH] = M[(a0 + t / CH) * r + a0 + t % CH];
+      if (rt < nb) B[rt][CH] = rdiag[a0 + rt];
+      double acc[SV_T];
 #pragma unroll
-    for (int t = 0; t < 32; ++t) acc[t] = 0.0;
-    for (int64_t q = a0 + nb + lane; q < r; q += 32) {
-      const double yq = y[q];
+      for (int t = 0; t < SV_T; ++t) acc[t] = 0.0;
+      const double* Mr = M + (a0 + sub * SV_T) * r;
+#pragma unroll 2
+      for (int64_t q = q0 + lane; q < q1; q += 32) {
+        const double yq = y[q];
 #pragma unroll
-      for (int t = 0; t < 32; ++t)
-        if (t < nb) acc[t] = fma(Lt[(a0 + t) * r + q], yq, acc[t]);
+        for (int t = 0; t < SV_T; ++t)
+          if (sub * SV_T + t < nb) acc[t] = fma(Mr[t * r + q], yq, acc[t]);
+      }
+      const double v8 = warp_sum8(acc, lane);
+      if ((lane & 3) == 0 && sub * SV_T + (lane >> 2) < nb) y[a0 + sub * SV_T + (lane >> 2)] -= v8;
+      row_sync();
+      if (sub == 0) {
+        double v = lane < nb ? y[a0 + lane] : 0.0;
+        for (int k = 0; k < nb; ++k) {
+          const int c = pass ? nb - 1 - k : k;
+          const double xc = __shfl_sync(0xffffffffu, v, c) * B[c][CH];
+          const bool open = pass ? lane < c : lane > c && lane < nb;
+          if (lane == c)
+            v = xc;
+          else if (open)
+            v -= B[lane][c] * xc;
+        }
+        if (lane < nb) {
+          y[a0 + lane] = v;
+          if (pass && i < n) A[i * r + a0 + lane] = v;
+        }
+      }
+      row_sync();
     }
-    double v = warp_transpose_sum(acc, lane);
-    v = lane < nb ? y[a0 + lane] - v : 0.0;
-    stage_block(Lt, rdiag, r, a0, nb, B, lane);
-    for (int c = nb - 1; c >= 0; --c) {
-      const double xc = __shfl_sync(0xffffffffu, v, c) * B[c][32];
-      if (lane == c) v = xc;
-      else if (lane < c) v -= B[lane][c] * xc;
-    }
-    if (lane < nb) {
-      y[a0 + lane] = v;
-      A[i * r + a0 + lane] = v;
-    }
-    __syncwarp();
   }
 }
 
@@ -485,7 +514,7 @@ grom_status gram_of(grom_als* s, int q, int64_t r) {
 }
 
 // MTTKRP of layout m (0, 1, 2) with factors P (middle index) and Q (inner
-// index) into s->mt (r x n).
+// index) into s->mt (r x n), enqueued; als_wait collects its time and errors.
 grom_status mttkrp(grom_als* s, int m, int fp, int fq, int64_t r) {
   const K2Plan pl = k2_plan(s->n, (int)r, s->sm_count);
   K2Args a{};
@@ -500,65 +529,93 @@ grom_status mttkrp(grom_als* s, int m, int fp, int fq, int64_t r) {
   a.ev0 = s->ev0;
   a.ev1 = s->ev1;
   GROM_CUDA_TRY(k2_launch(pl, &s->tmap[m], a, s->stream));
+  return GROM_OK;
+}
+
+// Waits for the stream; after an MTTKRP its time and the device error word,
+// after a factorisation (ok != nullptr) whether every pivot was positive.
+grom_status als_wait(grom_als* s, bool mttkrp_ran, bool* ok) {
+  int flags[2] = {0, 0};
+  GROM_CUDA_TRY(cudaMemcpyAsync(flags, s->err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+  if (ok) GROM_CUDA_TRY(cudaMemcpyAsync(flags + 1, s->flag, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
   GROM_CUDA_TRY(cudaStreamSynchronize(s->stream));
   float ms = 0.f;
-  GROM_CUDA_TRY(cudaEventElapsedTime(&ms, s->ev0, s->ev1));
-  s->mttkrp_ms += ms;
-  ++s->mttkrp_calls;
-  int flag = 0;
-  GROM_CUDA_TRY(cudaMemcpy(&flag, s->err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (flag & DEV_ERR_TIMEOUT) {
+  if (mttkrp_ran) {
+    GROM_CUDA_TRY(cudaEventElapsedTime(&ms, s->ev0, s->ev1));
+    s->mttkrp_ms += ms;
+    ++s->mttkrp_calls;
+  }
+  if (flags[0] & DEV_ERR_TIMEOUT) {
     cudaMemset(s->err, 0, sizeof(int));
     return fail(GROM_ERR_TIMEOUT, "grom_als_fit: a device-side wait timed out");
   }
+  if (ok) *ok = flags[1] == 0;
   return GROM_OK;
 }
 
-// Cholesky of s->h in place (lower); false if a pivot broke down.
-grom_status cholesky_dev(grom_als* s, int64_t r, bool* ok) {
-  GROM_CUDA_TRY(cudaMemsetAsync(s->flag, 0, sizeof(int), s->stream));
+// H = Ga o Gb + rel max diag(Ga o Gb) I and its Cholesky factor L (s->h) and
+// L^T (s->lt), on stream st.
+grom_status factorise(grom_als* s, const double* Ga, const double* Gb, int64_t r, double rel, cudaStream_t st) {
+  GROM_CUDA_TRY(cudaMemsetAsync(s->flag, 0, sizeof(int), st));
+  k_als_normal<<<grid_for(r * r), 256, 0, st>>>(Ga, Gb, r, rel, s->h);
   for (int64_t kb = 0; kb < r; kb += CH) {
-    k_chol_diag<<<1, CH * CH, 0, s->stream>>>(s->h, r, kb, s->rdiag, s->flag);
+    k_chol_diag<<<1, 128, 0, st>>>(s->h, r, kb, s->rdiag, s->flag);
     if (kb + CH < r) {
       const int64_t rows = r - kb - CH, m = (rows + UT - 1) / UT;
-      k_chol_panel<<<(unsigned)((rows + 7) / 8), 256, 0, s->stream>>>(s->h, r, kb, s->rdiag);
-      k_chol_update<<<(unsigned)(m * (m + 1) / 2), UT * UT, 0, s->stream>>>(s->h, r, kb);
+      k_chol_panel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(s->h, r, kb, s->rdiag);
+      k_chol_update<<<(unsigned)(m * (m + 1) / 2), UT * UT, 0, st>>>(s->h, r, kb);
     }
   }
+  k_transpose<<<grid_for(r * r), 256, 0, st>>>(s->h, r, s->lt);
   GROM_CUDA_TRY(cudaGetLastError());
-  int flag = 0;
-  GROM_CUDA_TRY(cudaMemcpyAsync(&flag, s->flag, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-  GROM_CUDA_TRY(cudaStreamSynchronize(s->stream));
-  *ok = flag == 0;
   return GROM_OK;
 }
 
-// The normal-equation update dst = M H^-1 (M = s->mt), H = Ga o Gb +
-// ridge max diag(Ga o Gb) I.  If H is numerically singular (ALS on a tensor
-// dominated by a few components drives the factor columns towards each
-// other), retry with an extra mu max diag I, mu = 1e-12 growing 100x up to
-// three times.
-grom_status ls_update(grom_als* s, const double* Ga, const double* Gb, int64_t r, double ridge, double* dst) {
-  const auto t0 = std::chrono::steady_clock::now();
-  const int64_t n = s->n;
-  bool ok = false;
-  double mu = 0.0;
+// dst = M H^-1 (M = s->mt) with the factors in s->h and s->lt.
+grom_status triangular_solves(grom_als* s, int64_t r, double* dst) {
+  const size_t smem = (size_t)SV_ROWS * r * sizeof(double);
+  if (smem > 12 * 1024)
+    GROM_CUDA_TRY(cudaFuncSetAttribute(k_als_rowsolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_als_rowsolve<<<(unsigned)((s->n + SV_ROWS - 1) / SV_ROWS), 32 * SV_ROWS * SV_WARPS, smem, s->stream>>>(
+      s->h, s->lt, s->rdiag, s->mt, s->n, r, dst);
+  GROM_CUDA_TRY(cudaGetLastError());
+  return GROM_OK;
+}
+
+// One least-squares update dst = M H^-1 for mode m with the other modes'
+// factors fp, fq: M by MTTKRP (unless s->mt already holds it), H = Ga o Gb +
+// ridge max diag(Ga o Gb) I factorised beside it.  If H is numerically
+// singular (ALS on a tensor dominated by a few components drives the factor
+// columns towards each other), retry with an extra mu max diag I, mu = 1e-12
+// growing 100x up to three times.
+grom_status ls_update(grom_als* s, int m, int fp, int fq, int64_t r, double ridge, double* dst, bool have_m) {
+  const double *Ga = s->gram[fp], *Gb = s->gram[fq];
   grom_status st;
+  GROM_CUDA_TRY(cudaEventRecord(s->fork, s->stream));
+  GROM_CUDA_TRY(cudaStreamWaitEvent(s->side, s->fork, 0));
+  if ((st = factorise(s, Ga, Gb, r, ridge, s->side))) return st;
+  GROM_CUDA_TRY(cudaEventRecord(s->join, s->side));
+  if (!have_m && (st = mttkrp(s, m, fp, fq, r))) return st;
+  GROM_CUDA_TRY(cudaEventRecord(s->sv0, s->stream));
+  GROM_CUDA_TRY(cudaStreamWaitEvent(s->stream, s->join, 0));
+  bool ok = false, ran = !have_m;
+  double mu = 0.0;
   for (int attempt = 0; attempt < 4 && !ok; ++attempt) {
-    k_als_normal<<<grid_for(r * r), 256, 0, s->stream>>>(Ga, Gb, r, ridge + mu, s->h);
-    if ((st = cholesky_dev(s, r, &ok))) return st;
-    mu = mu == 0.0 ? 1e-12 : mu * 100.0;
+    if (attempt > 0) {
+      mu = mu == 0.0 ? 1e-12 : mu * 100.0;
+      if ((st = factorise(s, Ga, Gb, r, ridge + mu, s->stream))) return st;
+    }
+    if ((st = triangular_solves(s, r, s->anew))) return st;
+    GROM_CUDA_TRY(cudaEventRecord(s->sv1, s->stream));
+    if ((st = als_wait(s, ran, &ok))) return st;
+    ran = false;
   }
   if (!ok) return fail(GROM_ERR_INVALID_ARG, "grom_als_fit: a Gram matrix is not positive definite");
-  k_transpose<<<grid_for(r * r), 256, 0, s->stream>>>(s->h, r, s->lt);
-  const size_t smem = (size_t)SOLVE_WARPS * (r + 32 * 33) * sizeof(double);
-  if (smem > 48 * 1024)
-    GROM_CUDA_TRY(cudaFuncSetAttribute(k_als_rowsolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_als_rowsolve<<<(unsigned)((n + SOLVE_WARPS - 1) / SOLVE_WARPS), 32 * SOLVE_WARPS, smem, s->stream>>>(
-      s->h, s->lt, s->rdiag, s->mt, n, r, dst);
-  GROM_CUDA_TRY(cudaGetLastError());
-  GROM_CUDA_TRY(cudaStreamSynchronize(s->stream));
-  s->solve_ms += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+  float ms = 0.f;
+  GROM_CUDA_TRY(cudaEventElapsedTime(&ms, s->sv0, s->sv1));
+  s->solve_ms += ms;
+  if (dst != s->anew)
+    GROM_CUDA_TRY(cudaMemcpyAsync(dst, s->anew, (size_t)(s->n * r) * sizeof(double), cudaMemcpyDeviceToDevice, s->stream));
   return GROM_OK;
 }
 
@@ -571,7 +628,7 @@ grom_status residual_of(grom_als* s, int64_t r, double* out) {
   GROM_CUDA_TRY(cudaGetLastError());
   double ph[2 * ALS_PARTS];
   GROM_CUDA_TRY(cudaMemcpyAsync(ph, s->part, sizeof(ph), cudaMemcpyDeviceToHost, s->stream));
-  GROM_CUDA_TRY(cudaStreamSynchronize(s->stream));
+  if (const grom_status st = als_wait(s, true, nullptr)) return st;
   double ip = 0.0, kk = 0.0;
   for (int q = 0; q < ALS_PARTS; ++q) {
     ip += ph[q];
@@ -621,7 +678,11 @@ grom_status grom_als_create(int32_t n, const double* tensor, void* stream, grom_
   }
   if (cudaMalloc(&s->err, sizeof(int)) != cudaSuccess || cudaMemsetAsync(s->err, 0, sizeof(int), s->stream) != cudaSuccess)
     return bail(fail(GROM_ERR_OOM, "grom_als_create: device allocation"));
-  if (cudaEventCreate(&s->ev0) != cudaSuccess || cudaEventCreate(&s->ev1) != cudaSuccess)
+  if (cudaEventCreate(&s->ev0) != cudaSuccess || cudaEventCreate(&s->ev1) != cudaSuccess ||
+      cudaEventCreate(&s->sv0) != cudaSuccess || cudaEventCreate(&s->sv1) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) != cudaSuccess)
     return bail(cuda_fail(cudaGetLastError(), "grom_als_create: events"));
   // stream the FP64 tensor through a staging buffer by test index
   const int64_t per_i = (int64_t)n * n;
@@ -685,9 +746,9 @@ grom_status grom_als_fit(grom_als* s, int32_t rank, int32_t method, int32_t iter
       for (int m = 0; m < 3; ++m) {
         // layout m: rows of mode m; P, Q = the factors of its middle and inner index
         const int fp = m == 0 ? 1 : 0, fq = m == 2 ? 1 : 2;
-        if ((st = mttkrp(s, m, fp, fq, r)) || (st = ls_update(s, s->gram[fp], s->gram[fq], r, ridge, s->f[m])) ||
-            (st = gram_of(s, m, r)))
-          return st;
+        // the residual's MTTKRP of the last iteration is this iteration's first
+        const bool have_m = m == 0 && it > 0 && residual;
+        if ((st = ls_update(s, m, fp, fq, r, ridge, s->f[m], have_m)) || (st = gram_of(s, m, r))) return st;
       }
       // <X, K> from a fresh mode-1 MTTKRP with the final factors: the M the
       // last update used carries the noise that update amplified along the
@@ -707,14 +768,14 @@ grom_status grom_als_fit(grom_als* s, int32_t rank, int32_t method, int32_t iter
     if ((st = gram_of(s, q, r))) return st;
   for (int it = 0; it < iters; ++it) {
     // A2 as in ALS (layout X2: P = A1, Q = A3), halves averaged
-    if ((st = mttkrp(s, 1, 0, 2, r)) || (st = ls_update(s, s->gram[0], s->gram[2], r, ridge, s->anew))) return st;
+    if ((st = ls_update(s, 1, 0, 2, r, ridge, s->anew, false))) return st;
     k_skew_halves<<<gh, 256, 0, s->stream>>>(s->anew, n, h, s->b1);
     k_skew_derive<<<gh, 256, 0, s->stream>>>(s->f[0], s->b1, n, h, s->f[1], nullptr);
     GROM_CUDA_TRY(cudaGetLastError());
     if ((st = gram_of(s, 1, r))) return st;
     for (int sub = 0; sub < subiters; ++sub) {
       // A1_next with A2, A3 fixed (layout X1: P = A2, Q = A3), then momentum
-      if ((st = mttkrp(s, 0, 1, 2, r)) || (st = ls_update(s, s->gram[1], s->gram[2], r, ridge, s->anew))) return st;
+      if ((st = ls_update(s, 0, 1, 2, r, ridge, s->anew, false))) return st;
       k_momentum<<<grid_for(n * r), 256, 0, s->stream>>>(s->f[0], s->anew, n * r, lambda);
       k_skew_derive<<<gh, 256, 0, s->stream>>>(s->f[0], s->b1, n, h, nullptr, s->f[2]);
       GROM_CUDA_TRY(cudaGetLastError());
@@ -738,9 +799,11 @@ grom_status grom_als_stats(grom_als* s, double* mttkrp_ms, int64_t* mttkrp_calls
 
 grom_status grom_als_destroy(grom_als* s) {
   if (!s) return GROM_OK;
+  if (s->side) cudaStreamSynchronize(s->side);
   if (s->stream) cudaStreamSynchronize(s->stream);
-  if (s->ev0) cudaEventDestroy(s->ev0);
-  if (s->ev1) cudaEventDestroy(s->ev1);
+  for (cudaEvent_t e : {s->ev0, s->ev1, s->sv0, s->sv1, s->fork, s->join})
+    if (e) cudaEventDestroy(e);
+  if (s->side) cudaStreamDestroy(s->side);
   for (auto p : s->x)
     if (p) cudaFree(p);
   als_free_fit(s);
