@@ -27,6 +27,7 @@ SOURCES = [
     "k3_ds.cu",
     "k3_oz.cu",
     "k3_persistent.cu",
+    "k3_exchange.cu",
     "k1_plan.cu",
     "k1_f64.cu",
     "k1_f32x2.cu",

@@ -220,7 +220,7 @@ static void rom_free(grom_rom* r) {
                   r->lin_diag, r->forcing, r->part, r->err,  r->k2_scratch, r->k3g_scratch, r->k3p_scratch,
                   r->k3t_factors, r->k3t_scratch, r->k3d_factors, r->k3d_scratch, r->k3o_factors, r->k3o_scratch,
                   r->k1p_dg, r->k1p_tg, r->probe, r->svd_ut, r->svd_sigma, r->svd_beta, r->k1pp_scratch,
-                  r->k2_tiles, r->k1t_scratch, r->k1t.d_off, r->k1t.d_ranges};
+                  r->k2_tiles, r->k3x_scratch, r->k1t_scratch, r->k1t.d_off, r->k1t.d_ranges};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (cudaEvent_t e : r->prof_ev) cudaEventDestroy(e);
@@ -738,7 +738,10 @@ grom_status grom_create(const grom_desc* d, void* stream, grom_rom** out) {
     // persistent stepper (its grid-barrier word starts at zero)
     const size_t kp = k3p_scratch_bytes(n, rp, r->storage, r->sm_count);
     if ((st = dmalloc(&r->k3p_scratch, kp, &r->total_bytes))) return bail(st);
-    if (cudaMemsetAsync(r->k3p_scratch, 0, kp, r->stream) != cudaSuccess)
+    const size_t kx = k3x_scratch_bytes(n, rp, r->sm_count);
+    if ((st = dmalloc(&r->k3x_scratch, kx, &r->total_bytes))) return bail(st);
+    if (cudaMemsetAsync(r->k3p_scratch, 0, kp, r->stream) != cudaSuccess ||
+        cudaMemsetAsync(r->k3x_scratch, 0, kx, r->stream) != cudaSuccess)
       return bail(cuda_fail(cudaGetLastError(), "grom_create"));
     // the per-tile arrival counters of the projection kernel start at zero
     if (cudaMemsetAsync(r->part, 0, r->part_bytes, r->stream) != cudaSuccess)
@@ -1274,15 +1277,22 @@ grom_status grom_step(grom_traj* t, int32_t nsteps, double* energy, double* inva
   if (nsteps < 0) return fail(GROM_ERR_INVALID_ARG, "grom_step: nsteps < 0");
   grom_rom* r = t->rom;
   if (!full_ready(r)) return fail(GROM_ERR_INVALID_ARG, "grom_step: tensor rows missing");
-  // CP forms with a few trajectories: all steps in one persistent launch
-  if (r->diagonal && is_cp(r) && r->k3p_scratch && !t->active && !r->prof &&
-      t->batch <= k3p_max_batch(r->storage) && nsteps >= 4 && !use_k3t(r, t->batch, false) &&
-      k3p_fits(r->n, r->k3.rb, r->storage, t->batch, r->sm_count)) {
-    StepArgs a = step_args(t, energy, invariant);
-    cudaError_t e = k3p_launch(r->op, r->op + r->panel_bytes, r->op + 2 * r->panel_bytes, r->form, r->n, r->k3.rb,
-                               r->storage, t->batch, nsteps, a, r->k3p_scratch, r->sm_count, r->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "grom_step persistent launch");
-    return GROM_OK;
+  // CP forms with a few trajectories: all steps in one persistent launch,
+  // without grid barriers where the factors fit shared memory by columns and
+  // by rows
+  if (r->diagonal && is_cp(r) && !t->active && !r->prof && nsteps >= 4 && !use_k3t(r, t->batch, false)) {
+    const uint8_t *fa = r->op, *fb = r->op + r->panel_bytes, *fc = r->op + 2 * r->panel_bytes;
+    const bool few = t->batch <= k3p_max_batch(r->storage);
+    const StepArgs a = step_args(t, energy, invariant);
+    cudaError_t e = cudaErrorNotSupported;
+    if (few && k3x_fits(r->n, r->k3.rb, r->form, r->storage, t->batch, r->sm_count))
+      e = k3x_launch(fa, fb, fc, r->form, r->n, r->k3.rb, r->storage, t->batch, nsteps, a, r->k3x_scratch, r->sm_count,
+                     r->stream);
+    else if (few && k3p_fits(r->n, r->k3.rb, r->storage, t->batch, r->sm_count))
+      e = k3p_launch(fa, fb, fc, r->form, r->n, r->k3.rb, r->storage, t->batch, nsteps, a, r->k3p_scratch, r->sm_count,
+                     r->stream);
+    if (e == cudaSuccess) return GROM_OK;
+    if (e != cudaErrorNotSupported) return cuda_fail(e, "grom_step persistent launch");
   }
   // full G-ROM with the skew-packed tensor and a few trajectories: all steps
   // in one persistent launch (falls back to the graphs below when the launch

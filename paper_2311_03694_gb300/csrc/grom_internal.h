@@ -318,6 +318,15 @@ cudaError_t k3p_launch(const uint8_t* fa, const uint8_t* fb, const uint8_t* fc, 
                        int storage, int batch, int nsteps, const StepArgs& st, void* scratch, int sm_count,
                        cudaStream_t s);
 
+// The same without grid barriers, for factors that fit shared memory by
+// columns and by rows (k3_exchange.cu).  scratch: k3x_scratch_bytes, zeroed
+// once at creation.
+size_t k3x_scratch_bytes(int64_t n, int64_t rp, int sm_count);
+bool k3x_fits(int64_t n, int64_t rp, int form, int storage, int batch, int sm_count);
+cudaError_t k3x_launch(const uint8_t* fa, const uint8_t* fb, const uint8_t* fc, int form, int64_t n, int64_t rp,
+                       int storage, int batch, int nsteps, const StepArgs& st, void* scratch, int sm_count,
+                       cudaStream_t s);
+
 // --------------------------------------------------------------- stepper
 struct StepArgs {
   int64_t n;
@@ -489,6 +498,7 @@ struct grom_rom {
   void* k3t_scratch = nullptr;
   CUtensorMap k3t_tmap_ft, k3t_tmap_ae;
   void* k3p_scratch = nullptr;       // persistent CP stepper: partials, h, barrier
+  void* k3x_scratch = nullptr;       // exchange CP stepper: published words
   size_t k2_scratch_bytes = 0;
   size_t k3t_scratch_bytes = 0;
   std::vector<grom_tuning> tuning;   // per batch bucket ceil(batch / 16); kernel 0: untuned
