@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(K1_THREADS, 1) k1_stream_kernel(const K1Plan p
   volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + K1_STAGES);
   uint8_t* ureg = reinterpret_cast<uint8_t*>(empty + K1_STAGES) + 16;
 
+  __shared__ double wsum[K1_CONSUMERS / 32][NB];  // pl.whole: the warps' sums of the CTA's test index
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t n = pl.n, np = pl.np, row_bytes = pl.row_bytes;
   const int64_t G = gridDim.x;
@@ -273,7 +274,10 @@ __global__ void __launch_bounds__(K1_THREADS, 1) k1_stream_kernel(const K1Plan p
         const int64_t seg = i_seg - first_i;
         double* dst = a.part + (((int64_t)blockIdx.x * pl.maxseg + seg) * (K1_CONSUMERS / 32) + warp) * NB;
 #pragma unroll
-        for (int b = 0; b < NB; ++b) dst[b] = contrib[b];
+        for (int b = 0; b < NB; ++b) {
+          dst[b] = contrib[b];
+          if (pl.whole) wsum[warp][b] = contrib[b];
+        }
       }
     };
 
@@ -432,6 +436,19 @@ __global__ void __launch_bounds__(K1_THREADS, 1) k1_stream_kernel(const K1Plan p
       }
     }
     if (cur_i >= 0 && !__any_sync(0xffffffffu, *abort_flag != 0)) flush(cur_i);
+    if (pl.whole && !a.skip_finalize) {
+      ptx::named_sync(1, K1_CONSUMERS);
+      if (tid < a.nb && !*abort_flag) {
+        const int bg = b0 + tid;
+        if (!a.active || a.active[bg]) {
+          double v = 0.0;
+#pragma unroll
+          for (int w = 0; w < K1_CONSUMERS / 32; ++w) v += wsum[w][tid];
+          double* dst = a.taken ? a.hist + bg * a.hist_stride + (3 + a.taken[bg] % 3) * n : a.c + bg * a.c_stride;
+          dst[first_i] = v;
+        }
+      }
+    }
   }
   __syncthreads();
 }
@@ -471,7 +488,7 @@ cudaError_t k1_launch_one(const K1Plan& pl, const K1Args& a, int b0, cudaStream_
   e = cudaGetLastError();
   if (e == cudaSuccess && a.ev1) e = prof_record(a.ev1, s);
   if (e != cudaSuccess) return e;
-  if (a.skip_finalize) return cudaSuccess;
+  if (a.skip_finalize || pl.whole) return cudaSuccess;
   const int64_t total = pl.n * a.nb;
   k1_finalize_kernel<NB><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(pl, a, b0);
   return cudaGetLastError();

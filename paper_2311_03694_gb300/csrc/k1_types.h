@@ -31,6 +31,7 @@ struct K1Plan {
   int64_t T;           // total chunks = n * cpi
   int grid;            // persistent CTAs
   int maxseg;          // max test-index segments per CTA
+  int whole;           // 1: every CTA covers one whole test index and finalises it itself (dense layout)
   int qm;              // vector positions per consumer thread per row (1,2,4,8)
   int nb_max;          // trajectories per pass
   size_t smem;         // dynamic shared memory
