@@ -26,6 +26,7 @@ SOURCES = [
     "k3_gemm.cu",
     "k3_ds.cu",
     "k3_oz.cu",
+    "k3_tri.cu",
     "k3_persistent.cu",
     "k3_exchange.cu",
     "k1_plan.cu",

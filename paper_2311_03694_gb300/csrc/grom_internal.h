@@ -41,6 +41,31 @@ inline cudaError_t prof_record(cudaEvent_t ev, cudaStream_t s) {
 constexpr int DEV_ERR_TIMEOUT = 1;
 constexpr int DEV_ERR_NONFINITE = 2;
 
+// Launches a kernel that may start while the one before it on the stream is
+// still running (programmatic dependent launch): it calls grid_wait() before
+// it touches anything the other wrote, so that its launch and set-up overlap.
+// Launched the plain way, the kernels' grid_wait and grid_trigger do nothing.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+// Until every kernel before this one has completed and its writes are visible.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The next kernel's CTAs may be launched once every CTA has called this.
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 // ------------------------------------------------------------- layout
 // The stored tensor pads the advected index k to np = round_up(n, 64) with
 // zeros, so every stored row starts on a 128-byte boundary for every
@@ -212,9 +237,9 @@ cudaError_t k3g_launch(const K3Plan& p, int storage, const K3Args& a, int batch,
 constexpr int K3G_MIN_BATCH = 16;
 // AUTO steps FP64 CP batches (16 trajectories and more) on the tensor cores
 // (K3O) from this much work per step (N R B) on, else with K3D (measured on
-// GB300: N = R = 1024 at 16 trajectories 0.063 against 0.085 ms, at 1024
-// 0.535 against 1.93 ms; 64 trajectories of N = 512, R = 256 0.035 against
-// 0.034 ms, of N = R = 256 0.031 against 0.023 ms)
+// GB300, us a step of K3O against K3D: N = R = 1024 at 1024 trajectories 457
+// against 1930; N = 512, R = 256 at 64 trajectories 32.3 against 33.2; N = R =
+// 512 at 32 33.9 against 33.1; N = R = 256 at 128 33.6 against 32.6)
 constexpr int64_t K3O_MIN_WORK = (int64_t)1 << 24;
 // Batched CP form of FP64 ROMs at FP64 tolerance in double-single FP32
 // arithmetic (K3D, same batch sizes as K3g): hi/lo copies of the factors
@@ -248,6 +273,10 @@ cudaError_t k3o_launch(int64_t n, int64_t rp, int64_t r, const K3Args& a, const 
 cudaError_t k3o_launch_step(int64_t n, int64_t rp, int64_t r, const K3Args& a, const void* factors, int batch,
                             void* scratch, int* err, int sm_count, const StepArgs& st, int step_index,
                             cudaStream_t s);
+// The slice products with all levels in one tile (k3_tri.cu): out holds [split][hi, lo][nslice][mslice].
+int k3o_tri_splits(int64_t mslice, int64_t nslice, int64_t K, int sm_count);
+cudaError_t k3o_tri_launch(const void* A, int64_t mslice, const void* B, int64_t nslice, int64_t K, float* out, int* err,
+                           int sm_count, cudaStream_t s);
 cudaError_t k3o_gemm_launch(const void* A, int64_t M, int64_t mslice, const void* B, int64_t ncols,
                             int64_t nslice, int64_t K, int slices, float* out, int* err, int sm_count,
                             cudaStream_t s);

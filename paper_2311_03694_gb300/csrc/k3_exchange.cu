@@ -23,7 +23,7 @@
 // barriers and partial sums (k3_persistent.cu, which keeps the larger ROMs);
 // n = r = 512 F64: 12.4 against 20.0; n = 256 F64, two trajectories: 14.2
 // against 40.1.  Of the 6.4 us the exchanges take 3.0 and the dependent
-// arithmetic (FP64 operations some 190 cycles apart) most of the rest.
+// arithmetic (FP64 operations some 70 cycles apart) most of the rest.
 // The sums of FP32 products are carried in three floats (ts_add) across
 // vectors and lanes, in place of the FP64 sums over the CTAs' partials.
 #include <algorithm>
@@ -184,6 +184,14 @@ __device__ __forceinline__ bool kx_poll(const unsigned long long* w, int count, 
   return true;
 }
 
+// A wait that ran out.  The base goes on as after a whole launch, so that the
+// words this one did publish are not taken for a later launch's.
+__device__ __forceinline__ void kx_abort(volatile int* abort_flag, int* err, unsigned int* base, uint32_t next) {
+  *abort_flag = 1;
+  *reinterpret_cast<volatile unsigned int*>(base) = next;
+  atomicOr(err, DEV_ERR_TIMEOUT);
+}
+
 template <int ST, int NB>
 __global__ void __launch_bounds__(KX_THREADS, 1) k3x_kernel(const KXArgs p) {
   using T = KXT<ST>;
@@ -291,8 +299,7 @@ __global__ void __launch_bounds__(KX_THREADS, 1) k3x_kernel(const KXArgs p) {
       uint32_t x[4];
       if (!kx_poll<false>(w + (size_t)q * NB * 4, 4, tag0 + 1u + (uint32_t)s, 0, 1, abort_flag,
                    [&](int k, uint32_t bits) { x[k] = bits; })) {
-        *abort_flag = 1;
-        atomicOr(st.err, DEV_ERR_TIMEOUT);
+        kx_abort(abort_flag, st.err, p.base, tag0 + 1u + (uint32_t)p.nsteps);
         break;
       }
       e += __hiloint2double((int)x[1], (int)x[0]);
@@ -331,10 +338,7 @@ __global__ void __launch_bounds__(KX_THREADS, 1) k3x_kernel(const KXArgs p) {
         reinterpret_cast<uint32_t*>(us)[(size_t)T::WORDS * (b * npad + kx_pos<ST>(i, npad)) + half] = bits;
       });
     }
-    if (!ok) {
-      *abort_flag = 1;
-      atomicOr(st.err, DEV_ERR_TIMEOUT);
-    }
+    if (!ok) kx_abort(abort_flag, st.err, p.base, tag0 + 1u + (uint32_t)p.nsteps);
     if (__syncthreads_or(*abort_flag)) return;
     // ---- 2: projections of the owned columns
     for (int c = warp; c < rb; c += KX_WARPS) {
@@ -389,10 +393,7 @@ __global__ void __launch_bounds__(KX_THREADS, 1) k3x_kernel(const KXArgs p) {
                                  hs)[(size_t)T::WORDS * ((which * NB + b) * rpad + kx_pos<ST>(r, rpad)) + half] = bits;
                            });
     }
-    if (!ok) {
-      *abort_flag = 1;
-      atomicOr(st.err, DEV_ERR_TIMEOUT);
-    }
+    if (!ok) kx_abort(abort_flag, st.err, p.base, tag0 + 1u + (uint32_t)p.nsteps);
     if (__syncthreads_or(*abort_flag)) return;
     // ---- 4: the owned rows
     double e_acc = 0.0, i_acc = 0.0;

@@ -16,11 +16,12 @@
 // emulation of the whole evaluation on the workload's factors gives 5.1e-15
 // per evaluation against FP64 at N = R = 1024 (1.2e-12 with S = 8; with
 // 7-bit digits, 2.7e-15 at S = 8, but exactness then holds only for K <=
-// 1024).  The projections of ROMs of N <= 1024 (K = N) therefore use eight
-// 7-bit digits (36 slice pairs, exact; 2.7e-15 in the emulation), the
-// expansion (K = 2R or R, up to 4096) the nine 6-bit ones.  The sums over
-// slice pairs run in double-single FP32 arithmetic (ds_arith.cuh) from the
-// smallest weights up.
+// 1024).  ROMs of N <= 1024 use eight 7-bit digits (36 slice pairs) for both
+// GEMMs, whose products k3_tri.cu forms level by level over at most 384 of the
+// summed index at a time, so that a level's sum over its slice pairs is exact
+// in FP32 whatever the length; the others nine 6-bit digits, one product per
+// slice pair.  The sums over levels, splits and slice pairs run in
+// double-single FP32 arithmetic (ds_arith.cuh) from the smallest weights up.
 //
 //   slice_states  per trajectory: the state's scale and digits        (B rows)
 //   gemm          D1 = [digits of V W U]^T x [digits of the states]   (tcgen05)
@@ -29,8 +30,8 @@
 //   slice_h       per trajectory: the scale and digits of [H1 H2]
 //   gemm          D2 = [digits of U, -W] x [digits of H]             (tcgen05)
 //   combine_exp   c per (b, i) from D2, FP64 into the output or the ring
-// The factor digits and scales are made once, at create.  The GEMM computes
-// only the 128 x 128 tiles that hold a slice pair of the triangle.
+// The factor digits and scales are made once, at create.  Only products of
+// the triangle are formed.
 #include <algorithm>
 
 #include <cuda_bf16.h>
@@ -43,10 +44,10 @@ namespace grom {
 
 constexpr int OZ_S = 9;     // slices per operand: 6-bit digits (exact for K <= 4096)
 constexpr int OZ_BITS = 6;
-constexpr int OZ_S7 = 8;    // projections of N <= 1024: 7-bit digits (exact for K <= 1024)
+constexpr int OZ_S7 = 8;    // ROMs of N <= 1024: 7-bit digits (k3_tri.cu)
 constexpr int OZ_BITS7 = 7;
 constexpr int64_t OZ_MAX_K = 4096;  // longest exact dot product of 6-bit digits
-constexpr int64_t OZ_MAX_K7 = 1024; // of 7-bit digits
+constexpr int64_t OZ_MAX_K7 = 1024; // longest projection of 7-bit digits
 
 static inline int64_t oz_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
@@ -61,6 +62,8 @@ struct ODims {
   int64_t nc;        // expansion GEMM columns: S bq rounded up to the GEMM's tile width (the rest unused)
   int sp;            // projection slices: OZ_S7 (7-bit digits) when nk <= OZ_MAX_K7, else OZ_S
   int64_t ncp;       // projection GEMM columns: sp bq rounded up likewise
+  bool tri;          // sp == OZ_S7: all levels of a tile at once (k3_tri.cu), eight 7-bit digits throughout
+  int se;            // expansion slices: OZ_S7 with tri, else OZ_S
   int batch;
 };
 
@@ -81,6 +84,8 @@ static ODims oz_dims(int64_t n, int64_t rp, int64_t r, int form, int batch) {
   d.sp = d.nk <= OZ_MAX_K7 ? OZ_S7 : OZ_S;
   d.ncp = oz_up((int64_t)d.sp * d.bq, 128);
   if (d.ncp >= 512) d.ncp = oz_up(d.ncp, 256);
+  d.tri = d.sp == OZ_S7;
+  d.se = d.tri ? OZ_S7 : OZ_S;
   d.batch = batch;
   return d;
 }
@@ -97,7 +102,7 @@ static OFactors oz_factor_layout(const ODims& d) {
   OFactors L{};
   L.aproj = 0;
   L.aexp = oz_round(2 * (size_t)d.sp * d.mp * d.nk);
-  L.sproj = L.aexp + oz_round(2 * (size_t)OZ_S * d.me * d.rk);
+  L.sproj = L.aexp + oz_round(2 * (size_t)d.se * d.me * d.rk);
   L.sexp = L.sproj + oz_round(4 * (size_t)d.mp);
   L.total = L.sexp + oz_round(4 * (size_t)d.me);
   return L;
@@ -244,6 +249,7 @@ __global__ void __launch_bounds__(256) k3o_build_proj(const uint8_t* op, size_t 
 }
 
 // Expansion row i: [fa_i | -fc_i] (skew) or fa_i (general) over the rank.
+template <int S, int BITS>
 __global__ void __launch_bounds__(256) k3o_build_exp(const uint8_t* op, size_t panel_bytes, const ODims d,
                                                      __nv_bfloat16* aexp, int* sexp) {
   __shared__ unsigned long long sh[33];
@@ -265,10 +271,10 @@ __global__ void __launch_bounds__(256) k3o_build_exp(const uint8_t* op, size_t p
   const int e = oz_exp_d(oz_block_max(mx, sh));
   if (threadIdx.x == 0) sexp[i] = e;
   for (int64_t k = threadIdx.x; k < d.rk; k += blockDim.x) {
-    __nv_bfloat16 dg[OZ_S];
-    oz_digits<OZ_S, OZ_BITS>(oz_fix_d<OZ_S * OZ_BITS>(val(k), e), dg);
+    __nv_bfloat16 dg[S];
+    oz_digits<S, BITS>(oz_fix_d<S * BITS>(val(k), e), dg);
 #pragma unroll
-    for (int p = 0; p < OZ_S; ++p) aexp[((int64_t)p * d.me + i) * d.rk + k] = dg[p];
+    for (int p = 0; p < S; ++p) aexp[((int64_t)p * d.me + i) * d.rk + k] = dg[p];
   }
 }
 
@@ -282,6 +288,8 @@ __global__ void __launch_bounds__(256) k3o_slice_states(const ODims d, const K3A
   __shared__ unsigned long long sh[33];
   const int b = blockIdx.x;
   const int64_t k0 = (int64_t)blockIdx.y * 256, k1 = k0 + 256 < d.nk ? k0 + 256 : d.nk;  // this CTA's digits
+  grid_trigger();
+  grid_wait();
   const bool on = b < d.batch && (a.active == nullptr || a.active[b]);
   const double* u = on ? (a.taken ? a.hist + b * a.hist_stride + (a.taken[b] % 3) * d.n : a.u + b * a.u_stride)
                        : nullptr;
@@ -330,6 +338,27 @@ __device__ __forceinline__ void oz_sum(const float* __restrict__ D, int64_t M, i
   }
 }
 
+// The pairs of one output from k3_tri.cu, [split][hi, lo][bq][M], in split order.
+__device__ __forceinline__ void oz_sum_tri(const float* __restrict__ D, int splits, int64_t M, int64_t bq, int b,
+                                           int64_t m, float& S, float& s) {
+  const int64_t plane = bq * M;
+  const float* p = D + (int64_t)b * M + m;
+  S = 0.f;
+  s = 0.f;
+  for (int q0 = 0; q0 < splits; q0 += 8) {  // eight splits' loads in flight
+    float v[8][2];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (q0 + k < splits) {
+        v[k][0] = __ldcg(p + (int64_t)(q0 + k) * 2 * plane);
+        v[k][1] = __ldcg(p + (int64_t)(q0 + k) * 2 * plane + plane);
+      }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (q0 + k < splits) ds_add(S, s, v[k][0], v[k][1]);
+  }
+}
+
 // (S, s) times 2^e, exactly (e in the FP32 exponent range).
 __device__ __forceinline__ void oz_scale_ds(float& S, float& s, int e) {
   const float f = __int_as_float((e + 127) << 23);
@@ -345,16 +374,21 @@ __device__ __forceinline__ void oz_scale_ds(float& S, float& s, int e) {
 template <int S, int BITS>
 __global__ void __launch_bounds__(192) k3o_combine_proj(const ODims d, const float* __restrict__ D1,
                                                         const int* __restrict__ sproj, const int* __restrict__ tau,
-                                                        float* Hh, float* Hl, unsigned int* hmax) {
+                                                        float* Hh, float* Hl, unsigned int* hmax, const int splits) {
   __shared__ float V[3][64][2];
   const int f = threadIdx.x >> 6, jl = threadIdx.x & 63;
   const int b = blockIdx.y;
   const int64_t j = (int64_t)blockIdx.x * 64 + jl;
   const int64_t M = S * d.mp;
+  grid_trigger();
+  grid_wait();
   if (f < d.nf && j < d.r) {
     const int64_t m = (int64_t)f * d.r + j;
     float hi, lo;
-    oz_sum<S, BITS>(D1, M, d.mp, d.bq, b, m, hi, lo);
+    if constexpr (S == OZ_S7)
+      oz_sum_tri(D1, splits, d.mp, d.bq, b, m, hi, lo);
+    else
+      oz_sum<S, BITS>(D1, M, d.mp, d.bq, b, m, hi, lo);
     oz_scale_ds(hi, lo, sproj[m] + tau[b]);
     V[f][jl][0] = hi;
     V[f][jl][1] = lo;
@@ -380,10 +414,13 @@ __global__ void __launch_bounds__(192) k3o_combine_proj(const ODims d, const flo
 // CTAs (b, chunk of 256), b < bq: the scale and digits of [H1 | H2] of
 // trajectory b.  The scale is twice the power of two above max |hi|, so that
 // hi + lo stays below it.
+template <int S, int BITS>
 __global__ void __launch_bounds__(256) k3o_slice_h(const ODims d, const K3Args a, const float* Hh, const float* Hl,
                                                    const unsigned int* hmax, __nv_bfloat16* bh, int* tau2) {
   const int b = blockIdx.x;
   const int64_t k0 = (int64_t)blockIdx.y * 256, k1 = k0 + 256 < d.rk ? k0 + 256 : d.rk;  // this CTA's digits
+  grid_trigger();
+  grid_wait();
   const bool on = b < d.batch && (a.active == nullptr || a.active[b]);
   const int e = on && hmax[b] ? oz_exp_f(hmax[b]) + 1 : 0;
   if (threadIdx.x == 0 && blockIdx.y == 0) tau2[b] = e;
@@ -393,26 +430,31 @@ __global__ void __launch_bounds__(256) k3o_slice_h(const ODims d, const K3Args a
     if (on && k < (int64_t)d.nt * d.r) {
       const int t = (int)(k / d.r);
       const int64_t x = t * hplane + (int64_t)b * d.r + (k - (int64_t)t * d.r);
-      Y = oz_fix_f<OZ_S * OZ_BITS>(Hh[x], e) + oz_fix_f<OZ_S * OZ_BITS>(Hl[x], e);
+      Y = oz_fix_f<S * BITS>(Hh[x], e) + oz_fix_f<S * BITS>(Hl[x], e);
     }
-    __nv_bfloat16 dg[OZ_S];
-    oz_digits<OZ_S, OZ_BITS>(Y, dg);
+    __nv_bfloat16 dg[S];
+    oz_digits<S, BITS>(Y, dg);
 #pragma unroll
-    for (int p = 0; p < OZ_S; ++p) bh[((int64_t)p * d.bq + b) * d.rk + k] = dg[p];
+    for (int p = 0; p < S; ++p) bh[((int64_t)p * d.bq + b) * d.rk + k] = dg[p];
   }
 }
 
 // One thread per (b, i), i fastest: c_bi into the output or the ring.
 __global__ void __launch_bounds__(256) k3o_combine_exp(const ODims d, const K3Args a, const float* __restrict__ D2,
-                                                       const int* __restrict__ sexp, const int* __restrict__ tau2) {
+                                                       const int* __restrict__ sexp, const int* __restrict__ tau2,
+                                                       const int splits) {
   const int64_t total = (int64_t)d.batch * d.n;
   const int64_t M = OZ_S * d.me;
+  grid_wait();
   for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < total; o += (int64_t)gridDim.x * blockDim.x) {
     const int b = (int)(o / d.n);
     const int64_t i = o - (int64_t)b * d.n;
     if (a.active && !a.active[b]) continue;
     float S, s;
-    oz_sum<OZ_S, OZ_BITS>(D2, M, d.me, d.bq, b, i, S, s);
+    if (splits)
+      oz_sum_tri(D2, splits, d.me, d.bq, b, i, S, s);
+    else
+      oz_sum<OZ_S, OZ_BITS>(D2, M, d.me, d.bq, b, i, S, s);
     oz_scale_ds(S, s, sexp[i] + tau2[b]);
     double* dst = a.taken ? a.hist + b * a.hist_stride + (3 + a.taken[b] % 3) * d.n : a.c + b * a.c_stride;
     dst[i] = (double)S + (double)s;
@@ -428,11 +470,13 @@ __global__ void __launch_bounds__(256) k3o_combine_exp(const ODims d, const K3Ar
 template <bool PLAIN>
 __global__ void __launch_bounds__(STEP_MC_THREADS)
     k3o_exp_step(const ODims d, const float* __restrict__ D2, const int* __restrict__ sexp,
-                 const int* __restrict__ tau2, const StepArgs st, const int step_index) {
+                 const int* __restrict__ tau2, const int splits, const StepArgs st, const int step_index) {
   __shared__ double sh[64];
   __shared__ int bad;
   __shared__ int last;
   const int blk = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+  grid_trigger();
+  grid_wait();
   if (!st.active || st.active[b]) {
     const int64_t M = OZ_S * d.me;
     double* ring = st.hist + b * st.hist_stride + (3 + st.taken[b] % 3) * d.n;
@@ -440,7 +484,10 @@ __global__ void __launch_bounds__(STEP_MC_THREADS)
       const int64_t i = ((int64_t)blk * st.ept + e) * STEP_MC_THREADS + tid;
       if (i >= d.n) break;
       float S, s;
-      oz_sum<OZ_S, OZ_BITS>(D2, M, d.me, d.bq, b, i, S, s);
+      if (splits)
+        oz_sum_tri(D2, splits, d.me, d.bq, b, i, S, s);
+      else
+        oz_sum<OZ_S, OZ_BITS>(D2, M, d.me, d.bq, b, i, S, s);
       oz_scale_ds(S, s, sexp[i] + tau2[b]);
       ring[i] = (double)S + (double)s;
     }
@@ -474,8 +521,12 @@ cudaError_t k3o_build_factors(const uint8_t* op, size_t panel_bytes, int64_t n, 
     k3o_build_proj<OZ_S7, OZ_BITS7><<<(unsigned)d.mp, 256, 0, s>>>(op, panel_bytes, d, ap, sp);
   else
     k3o_build_proj<OZ_S, OZ_BITS><<<(unsigned)d.mp, 256, 0, s>>>(op, panel_bytes, d, ap, sp);
-  k3o_build_exp<<<(unsigned)d.me, 256, 0, s>>>(op, panel_bytes, d, reinterpret_cast<__nv_bfloat16*>(base + L.aexp),
-                                               reinterpret_cast<int*>(base + L.sexp));
+  auto* se = reinterpret_cast<int*>(base + L.sexp);
+  auto* ae = reinterpret_cast<__nv_bfloat16*>(base + L.aexp);
+  if (d.tri)
+    k3o_build_exp<OZ_S7, OZ_BITS7><<<(unsigned)d.me, 256, 0, s>>>(op, panel_bytes, d, ae, se);
+  else
+    k3o_build_exp<OZ_S, OZ_BITS><<<(unsigned)d.me, 256, 0, s>>>(op, panel_bytes, d, ae, se);
   return cudaGetLastError();
 }
 
@@ -489,7 +540,7 @@ static unsigned oz_flat_blocks(int64_t count, int sm_count) {
 // slice products in d2); returns d2 and the expansion scales.
 static cudaError_t k3o_front(const ODims& d, const K3Args& a, const void* factors, void* scratch, int* err,
                              int sm_count, cudaStream_t s, const float** d2_out, const int** sexp_out,
-                             const int** tau2_out) {
+                             const int** tau2_out, int* splits2) {
   const OFactors F = oz_factor_layout(d);
   const OScratch L = oz_scratch_layout(d);
   const uint8_t* fb = static_cast<const uint8_t*>(factors);
@@ -505,23 +556,31 @@ static cudaError_t k3o_front(const ODims& d, const K3Args& a, const void* factor
   auto* d2 = reinterpret_cast<float*>(sb + L.d2);
   const dim3 gs((unsigned)d.bq, (unsigned)((d.nk + 255) / 256)), gc((unsigned)((d.r + 63) / 64), (unsigned)d.batch);
   const int* spj = reinterpret_cast<const int*>(fb + F.sproj);
-  if (d.sp == OZ_S7)
-    k3o_slice_states<OZ_S7, OZ_BITS7><<<gs, 256, 0, s>>>(d, a, bst, tau, hmax);
-  else
-    k3o_slice_states<OZ_S, OZ_BITS><<<gs, 256, 0, s>>>(d, a, bst, tau, hmax);
-  cudaError_t e = k3o_gemm_launch(fb + F.aproj, (int64_t)d.sp * d.mp, d.mp, bst, d.ncp, d.bq, d.nk, d.sp, d1, err,
-                                  sm_count, s);
-  if (e != cudaSuccess) return e;
-  if (d.sp == OZ_S7)
-    k3o_combine_proj<OZ_S7, OZ_BITS7><<<gc, 192, 0, s>>>(d, d1, spj, tau, hh, hl, hmax);
-  else
-    k3o_combine_proj<OZ_S, OZ_BITS><<<gc, 192, 0, s>>>(d, d1, spj, tau, hh, hl, hmax);
-  k3o_slice_h<<<dim3((unsigned)d.bq, (unsigned)((d.rk + 255) / 256)), 256, 0, s>>>(d, a, hh, hl, hmax, bh, tau2);
-  e = k3o_gemm_launch(fb + F.aexp, OZ_S * d.me, d.me, bh, d.nc, d.bq, d.rk, OZ_S, d2, err, sm_count, s);
   *d2_out = d2;
   *sexp_out = reinterpret_cast<const int*>(fb + F.sexp);
   *tau2_out = tau2;
-  return e;
+  *splits2 = 0;
+  const dim3 gh((unsigned)d.bq, (unsigned)((d.rk + 255) / 256));
+  if (d.tri) {
+    // each later kernel set up while the one before it runs: small batches are six launches of 2 to 8 us a step
+    const int s1 = k3o_tri_splits(d.mp, d.bq, d.nk, sm_count);
+    *splits2 = k3o_tri_splits(d.me, d.bq, d.rk, sm_count);
+    k3o_slice_states<OZ_S7, OZ_BITS7><<<gs, 256, 0, s>>>(d, a, bst, tau, hmax);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = k3o_tri_launch(fb + F.aproj, d.mp, bst, d.bq, d.nk, d1, err, sm_count, s);
+    if (e == cudaSuccess)
+      e = launch_dependent(k3o_combine_proj<OZ_S7, OZ_BITS7>, gc, 192, 0, s, d, d1, spj, tau, hh, hl, hmax, s1);
+    if (e == cudaSuccess)
+      e = launch_dependent(k3o_slice_h<OZ_S7, OZ_BITS7>, gh, 256, 0, s, d, a, hh, hl, hmax, bh, tau2);
+    return e == cudaSuccess ? k3o_tri_launch(fb + F.aexp, d.me, bh, d.bq, d.rk, d2, err, sm_count, s) : e;
+  }
+  k3o_slice_states<OZ_S, OZ_BITS><<<gs, 256, 0, s>>>(d, a, bst, tau, hmax);
+  cudaError_t e = k3o_gemm_launch(fb + F.aproj, (int64_t)d.sp * d.mp, d.mp, bst, d.ncp, d.bq, d.nk, d.sp, d1, err,
+                                  sm_count, s);
+  if (e != cudaSuccess) return e;
+  k3o_combine_proj<OZ_S, OZ_BITS><<<gc, 192, 0, s>>>(d, d1, spj, tau, hh, hl, hmax, 0);
+  k3o_slice_h<OZ_S, OZ_BITS><<<gh, 256, 0, s>>>(d, a, hh, hl, hmax, bh, tau2);
+  return k3o_gemm_launch(fb + F.aexp, OZ_S * d.me, d.me, bh, d.nc, d.bq, d.rk, OZ_S, d2, err, sm_count, s);
 }
 
 cudaError_t k3o_launch(int64_t n, int64_t rp, int64_t r, const K3Args& a, const void* factors, int batch,
@@ -529,9 +588,12 @@ cudaError_t k3o_launch(int64_t n, int64_t rp, int64_t r, const K3Args& a, const 
   const ODims d = oz_dims(n, rp, r, a.form, batch);
   const float* d2;
   const int *sexp, *tau2;
-  cudaError_t e = k3o_front(d, a, factors, scratch, err, sm_count, s, &d2, &sexp, &tau2);
+  int s2;
+  cudaError_t e = k3o_front(d, a, factors, scratch, err, sm_count, s, &d2, &sexp, &tau2, &s2);
   if (e != cudaSuccess) return e;
-  k3o_combine_exp<<<oz_flat_blocks((int64_t)batch * d.n, sm_count), 256, 0, s>>>(d, a, d2, sexp, tau2);
+  const unsigned blocks = oz_flat_blocks((int64_t)batch * d.n, sm_count);
+  if (s2) return launch_dependent(k3o_combine_exp, dim3(blocks), 256, 0, s, d, a, d2, sexp, tau2, s2);
+  k3o_combine_exp<<<blocks, 256, 0, s>>>(d, a, d2, sexp, tau2, s2);
   return cudaGetLastError();
 }
 
@@ -541,17 +603,21 @@ cudaError_t k3o_launch_step(int64_t n, int64_t rp, int64_t r, const K3Args& a, c
   const ODims d = oz_dims(n, rp, r, a.form, batch);
   const float* d2;
   const int *sexp, *tau2;
-  cudaError_t e = k3o_front(d, a, factors, scratch, err, sm_count, s, &d2, &sexp, &tau2);
+  int s2;
+  cudaError_t e = k3o_front(d, a, factors, scratch, err, sm_count, s, &d2, &sexp, &tau2, &s2);
   if (e != cudaSuccess) return e;
-  // one element per thread: each carries a 45-pair combine before its step
+  // one element per thread: each carries a combine of up to 45 pairs before its step
   StepArgs st1 = st;
   st1.ept = 1;
   st1.nblk = step_mc_blocks(n);
   const dim3 grid((unsigned)st1.nblk, (unsigned)batch);
+  if (s2)
+    return step_plain(st1) ? launch_dependent(k3o_exp_step<true>, grid, STEP_MC_THREADS, 0, s, d, d2, sexp, tau2, s2, st1, step_index)
+                           : launch_dependent(k3o_exp_step<false>, grid, STEP_MC_THREADS, 0, s, d, d2, sexp, tau2, s2, st1, step_index);
   if (step_plain(st1))
-    k3o_exp_step<true><<<grid, STEP_MC_THREADS, 0, s>>>(d, d2, sexp, tau2, st1, step_index);
+    k3o_exp_step<true><<<grid, STEP_MC_THREADS, 0, s>>>(d, d2, sexp, tau2, s2, st1, step_index);
   else
-    k3o_exp_step<false><<<grid, STEP_MC_THREADS, 0, s>>>(d, d2, sexp, tau2, st1, step_index);
+    k3o_exp_step<false><<<grid, STEP_MC_THREADS, 0, s>>>(d, d2, sexp, tau2, s2, st1, step_index);
   return cudaGetLastError();
 }
 

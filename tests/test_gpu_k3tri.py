@@ -1,0 +1,43 @@
+"""K3O's level-by-level slice products (k3_tri.cu) at the edges of their column
+tiles and summed ranges, and the one-product-per-pair form that N > 1024 keeps,
+against the FP64 oracle within the FP64 tolerance (1e-12)."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+import paper_2311_03694_gb300 as grom  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _factors(form, n, r, seed):
+    if form == "cp_skew":
+        U, V, W, _, _ = synth.cp_workload(n, r, 1)
+        return (U, V, W), lambda u: oracle.nonlinear_cp_skew(U, V, W, u)
+    rng = np.random.default_rng(seed)
+    A, B, C = (rng.standard_normal((n, r)) / np.sqrt(r) for _ in range(3))
+    return (A, B, C), lambda u: oracle.nonlinear_cp(A, B, C, u)
+
+
+@pytest.mark.parametrize("form", ["cp_skew", "cp"])
+@pytest.mark.parametrize("n,r,batch", [(64, 130, 64), (129, 64, 65), (400, 449, 16), (1024, 40, 33), (100, 1500, 16), (1030, 40, 16)])
+def test_k3o_level_products_at_tile_edges(form, n, r, batch):
+    # one and several column tiles, K ranges of one to six steps a CTA, of a
+# remainder step, and of many splits (rank 1500: 47 steps over 32 at most)
+    grom.build()
+    fac, ref = _factors(form, n, r, 900 + n)
+    rom = grom.Rom(n, form, "f64", factors=fac, stiffness=synth.diag_stiffness(n), max_batch=batch)
+    rom.set_kernel("tensor")
+    U = synth.initial_condition(n, 31 + n, 0, batch)
+    u = torch.from_numpy(U).cuda()
+    c = torch.full_like(u, float("nan"))
+    rom.nonlinear(u, c)
+    torch.cuda.synchronize()
+    got = c.cpu().numpy()
+    for b in (0, batch // 2, batch - 1):
+        want = ref(U[b])
+        assert np.linalg.norm(got[b] - want) <= 1e-12 * np.linalg.norm(want), (n, r, b)
+    rom.close()
