@@ -234,13 +234,13 @@ int64_t grom_rom_bytes(const grom_rom* rom);
  * (per-evaluation error ~1e-13 against FP64) with K3D: the projections and
  * the expansion as double-single FP32 GEMMs (every operand a hi/lo FP32 pair,
  * error-free products and sums) on hi/lo copies of the factors made at
- * create; from N R B >= 2^24 on (N modes, R rank, B trajectories), and with
- * GROM_KERNEL_TENSOR, with K3O: every operand split into integer digit
- * slices (eight of 7 bits for the projections of ROMs with N <= 1024, else
- * nine of 6 bits), the slice products on the tcgen05 tensor cores (exact in
- * FP32 for dot products of up to 1024 and 4096 terms respectively, so N and
- * the expansion's 2R (skew) or R at most 4096) and the slice pairs summed in
- * double-single arithmetic. */
+ * create; where it is faster (from N R B = 2^23 on with N R >= 2^19, else from
+ * 3 2^22, or 2^24 with small factors; N modes, R rank, B trajectories), and
+ * with GROM_KERNEL_TENSOR, with K3O: every operand split into integer digit
+ * slices (eight of 7 bits for ROMs with N <= 1024, else nine of 6 bits), the
+ * slice products on the tcgen05 tensor cores (sums exact in FP32; N and the
+ * expansion's 2R (skew) or R at most 4096) and summed in double-single
+ * arithmetic. */
 #define GROM_KERNEL_AUTO 0
 #define GROM_KERNEL_STREAM 1 /* K1: SIMT streaming kernel, up to 8 trajectories per pass, one
                                 launch per step (no persistent stepper); CP forms: the SIMT

@@ -236,11 +236,23 @@ cudaError_t k3g_launch(const K3Plan& p, int storage, const K3Args& a, int batch,
                        int sm_count, cudaStream_t s);
 constexpr int K3G_MIN_BATCH = 16;
 // AUTO steps FP64 CP batches (16 trajectories and more) on the tensor cores
-// (K3O) from this much work per step (N R B) on, else with K3D (measured on
-// GB300, us a step of K3O against K3D: N = R = 1024 at 1024 trajectories 457
-// against 1930; N = 512, R = 256 at 64 trajectories 32.3 against 33.2; N = R =
-// 512 at 32 33.9 against 33.1; N = R = 256 at 128 33.6 against 32.6)
-constexpr int64_t K3O_MIN_WORK = (int64_t)1 << 24;
+// (K3O) from this much work per step (N R B) on, earlier where the factors are
+// large (few trajectories leave K3D's 64-column tiles mostly empty), else with
+// K3D.  Measured on GB300, us a step of K3O against K3D, skew form: N = R =
+// 1024 at 1024 trajectories 457 against 1930; R = 512 at 16 36.9 against 53.3;
+// R = 256 at 48 31.6 against 52.6, at 32 32.6 against 34.4; N = R = 512 at 48
+// 33.3 against 53.1, at 32 33.9 against 33.1; N = R = 128 at 768 39.0 against
+// 42.2.  General form (three products where the skew form has five): N = 1024,
+// R = 512 at 16 30.5 against 35.7; N = R = 512 at 48 32.4 against 35.6; N =
+// 512, R = 256 at 96 32.6 against 31.1; N = 128, R = 64 at 1600 45.3 against
+// 39.5.
+inline bool k3o_faster(int64_t n, int64_t r, int64_t batch, bool skew) {
+  const int64_t nr = n * r;
+  int64_t least = (int64_t)1 << 24;
+  if (nr >= (int64_t)1 << (skew ? 14 : 18)) least = (int64_t)3 << 22;
+  if (nr >= (int64_t)1 << 19) least = (int64_t)1 << 23;
+  return nr * batch >= least;
+}
 // Batched CP form of FP64 ROMs at FP64 tolerance in double-single FP32
 // arithmetic (K3D, same batch sizes as K3g): hi/lo copies of the factors
 // made at create, then per step a state split and two GEMMs.

@@ -25,8 +25,8 @@ def _factors(form, n, r, seed):
 @pytest.mark.parametrize("form", ["cp_skew", "cp"])
 @pytest.mark.parametrize("n,r,batch", [(64, 130, 64), (129, 64, 65), (400, 449, 16), (1024, 40, 33), (100, 1500, 16), (1030, 40, 16)])
 def test_k3o_level_products_at_tile_edges(form, n, r, batch):
-    # one and several column tiles, K ranges of one to six steps a CTA, of a
-# remainder step, and of many splits (rank 1500: 47 steps over 32 at most)
+    # one and several column tiles, summed ranges of one to six steps a CTA,
+    # with a shorter last one and over many CTAs (rank 1500: 47 steps, skew)
     grom.build()
     fac, ref = _factors(form, n, r, 900 + n)
     rom = grom.Rom(n, form, "f64", factors=fac, stiffness=synth.diag_stiffness(n), max_batch=batch)
@@ -41,3 +41,30 @@ def test_k3o_level_products_at_tile_edges(form, n, r, batch):
         want = ref(U[b])
         assert np.linalg.norm(got[b] - want) <= 1e-12 * np.linalg.norm(want), (n, r, b)
     rom.close()
+
+
+@pytest.mark.parametrize("form,n,r,batch,tensor", [
+    ("cp_skew", 1024, 512, 16, True), ("cp", 1024, 512, 16, True),     # N R = 2^19 from 2^23 on
+    ("cp_skew", 1024, 448, 16, False), ("cp", 1024, 448, 16, False),   # below it: double-single
+    ("cp_skew", 128, 128, 768, True), ("cp", 128, 128, 768, False),    # 3 2^22
+])
+def test_k3o_rule_takes_the_path_it_states(form, n, r, batch, tensor):
+    # the default choice gives the bits of the path that its rule names, at FP64 tolerance
+    grom.build()
+    fac, ref = _factors(form, n, r, 77)
+    U = synth.initial_condition(n, 5, 0, batch)
+    rom = grom.Rom(n, form, "f64", factors=fac, stiffness=synth.diag_stiffness(n), max_batch=batch)
+    u = torch.from_numpy(U).cuda()
+    got = []
+    for kernel in ("auto", "tensor"):
+        rom.set_kernel(kernel)
+        c = torch.empty_like(u)
+        rom.nonlinear(u, c)
+        torch.cuda.synchronize()
+        got.append(c.cpu().numpy())
+    rom.close()
+    assert np.array_equal(got[0], got[1]) == tensor
+    for b in (0, batch - 1):
+        want = ref(U[b])
+        for c in got:
+            assert np.linalg.norm(c[b] - want) <= 1e-12 * np.linalg.norm(want), b
