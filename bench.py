@@ -493,6 +493,15 @@ def _row_len(n, layout):
     return _packed_len(n) if layout == "skew_packed" else (n + 63) // 64 * 64
 
 
+def _stored_bytes(n, layout, storage):
+    """Bytes of the stored full tensor, which one evaluation streams: N * N rows
+    (dense, and skew-packed BF16 and FP32), or for skew-packed F64 and F32X2
+    the folded layout, m + 1 rows of m values (a multiple of 16) for every m < N."""
+    if layout == "skew_packed" and storage in ("f64", "f32x2"):
+        return float(sum((m + 1) * ((m + 15) // 16 * 128) for m in range(1, n)))
+    return float(n) * n * _row_len(n, layout) * STORAGE_BYTES[storage]
+
+
 STORAGE_NAME = {"f32x2": "F32X2", "f64": "F64", "f32": "F32", "bf16": "BF16"}
 ARITH = {"f32x2": "F32X2 tensor (FP32 hi/lo pair, 48-bit significand), double-single FP32 contraction "
                   "(error-free products and sums), FP64 state; FP64 tolerance (1e-12 per evaluation)",
@@ -513,7 +522,7 @@ def _config(n, rank, layout, storage):
     return {"workload": _workload(n, rank), "storage": "%s; %s" % (ARITH[storage], how),
             "n": n, "cp_rank": rank, "batch_per_gpu": 1, "nu": NU, "dt": DT, "layout": layout,
             "l2": "inputs larger than L2 (stored tensor %.2f GB per step)" % (
-                n * n * _row_len(n, layout) * STORAGE_BYTES[storage] / 1e9)}
+                _stored_bytes(n, layout, storage) / 1e9)}
 
 
 # -------------------------------------------------------------------- main
@@ -590,14 +599,12 @@ def main():
     rom.profile(False)
 
     # roofline of the dominant kernel.  Its algorithmic bytes are the stored
-    # tensor per step, N * N rows of round_up(N/2, 64) (skew-packed) or
-    # round_up(N, 64) (dense) values of the storage type (8 bytes for F32X2
-    # and FP64, 4 for FP32, 2 for BF16), times the steps one launch runs:
-    # the persistent stepper runs all K steps (streaming, finalize and step)
-    # in one launch, the graph path one streaming launch per step.
+    # tensor per step (_stored_bytes), times the steps one launch runs: the
+    # persistent stepper runs all K steps (streaming, finalize and step) in
+    # one launch, the graph path one streaming launch per step.
     k1_avg_ms = k1_ms / max(1, k1_launches)
     steps_per_launch = args.steps // max(1, k1_launches)
-    step_bytes = float(n) * n * _row_len(n, args.layout) * STORAGE_BYTES[args.storage]
+    step_bytes = _stored_bytes(n, args.layout, args.storage)
     alg_bytes = step_bytes * steps_per_launch
     achieved = alg_bytes / (k1_avg_ms * 1e-3) / 1e9
     persistent = steps_per_launch > 1
@@ -606,8 +613,9 @@ def main():
     stname = STORAGE_NAME[args.storage]
     roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                 "frac": achieved / hbm_peak, "traffic": traffic * steps_per_launch if traffic else None,
-                "kernel": ("k1pp_kernel<%s> (persistent stepper: streaming, finalize and BDF3/EXT3 step of "
-                           "%d steps in one launch)" % (stname, steps_per_launch)) if persistent
+                "kernel": ("%s_kernel<%s> (persistent stepper: streaming, finalize and BDF3/EXT3 step of "
+                           "%d steps in one launch)" % ("k1t" if args.storage in ("f64", "f32x2") else "k1pp", stname,
+                                                        steps_per_launch)) if persistent
                 else "%s_kernel<%s> (finalize excluded)" % (kname, stname), "peak_kind": peak_kind,
                 "kernel_ms": k1_avg_ms, "kernel_launches": k1_launches, "steps_per_launch": steps_per_launch,
                 "algorithmic_bytes_per_launch": alg_bytes,
@@ -875,10 +883,10 @@ def main():
                     "ms_per_step": cms, "trajectory_steps_per_s": B * 1e3 / cms,
                     "alg_tflops": cflops / (cms * 1e-3) / 1e12,
                     "kernel": ("k3t_gemm x2 (tcgen05 projections and expansion)" if storage == "bf16" and B >= 16
-                               else ("k3o (tcgen05 GEMMs of digit slices: %s-bit for the projections, 6-bit for the "
-                                     "expansion; FP64 tolerance)" % ("7" if n <= 1024 else "6"))
+                               else "k3o (tcgen05 products of %s-bit digit slices; FP64 tolerance)" % (
+                                   "7" if n <= 1024 else "6")
                                if storage == "f64" and B >= 16 and (kernel == "tensor" or (
-                                   kernel == "auto" and n * R * B >= 2 ** 24))
+                                   kernel == "auto" and n * R * B >= (2 ** 23 if n * R >= 2 ** 19 else 3 * 2 ** 22)))
                                else "k3d project/expand (double-single FP32 GEMMs, FP64 tolerance)"
                                if storage == "f64" and kernel == "auto" and B >= 16
                                else "k3g project/expand (register-tiled FP64 GEMMs)" if B >= 16
