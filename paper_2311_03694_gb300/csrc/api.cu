@@ -300,6 +300,14 @@ static bool use_k3o(const grom_rom* r, int batch) {
   return r->kernel_choice == GROM_KERNEL_AUTO && k3o_faster(r->n, r->rank, batch, r->form == GROM_FORM_CP_SKEW);
 }
 
+// Evaluations of a few trajectories of FP64 factors in one launch
+// (k3_exchange.cu) in place of K3's two.  FP32 and BF16 factors keep K3: their
+// FP32 sums would be taken in another order.
+static bool use_k3x_eval(const grom_rom* r, int batch) {
+  return is_cp(r) && r->storage == GROM_F64 && r->kernel_choice == GROM_KERNEL_AUTO &&
+         k3x_eval_faster(r->n, r->k3.rb, r->form, batch, r->sm_count);
+}
+
 // K3T: the batched CP form on the tensor cores (BF16 factors)
 static bool use_k3t(const grom_rom* r, int batch, bool use_tuning = true) {
   if (!is_cp(r) || !r->k3t_factors) return false;
@@ -977,6 +985,7 @@ grom_status grom_nonlinear(grom_rom* r, int32_t batch, const double* u, double* 
         : use_k3d(r, batch) ? k3d_launch(r->k3, a, r->k3d_factors, batch, r->max_batch, r->k3d_scratch, r->sm_count,
                                          r->stream)
         : use_k3g(r, batch) ? k3g_launch(r->k3, r->storage, a, batch, r->max_batch, r->k3g_scratch, r->sm_count, r->stream)
+        : use_k3x_eval(r, batch) ? k3x_eval_launch(a, r->n, r->k3.rb, batch, r->k3x_scratch, r->err, r->sm_count, r->stream)
                             : k3_launch(r->k3, r->storage, a, batch, r->stream);
     if (e1) prof_record(e1, r->stream);
   }

@@ -367,6 +367,10 @@ bool k3x_fits(int64_t n, int64_t rp, int form, int storage, int batch, int sm_co
 cudaError_t k3x_launch(const uint8_t* fa, const uint8_t* fb, const uint8_t* fc, int form, int64_t n, int64_t rp,
                        int storage, int batch, int nsteps, const StepArgs& st, void* scratch, int sm_count,
                        cudaStream_t s);
+// One evaluation of FP64 factors the same way (scratch as above), and whether it beats k3_launch's two kernels.
+bool k3x_eval_faster(int64_t n, int64_t rp, int form, int batch, int sm_count);
+cudaError_t k3x_eval_launch(const K3Args& a, int64_t n, int64_t rp, int batch, void* scratch, int* err, int sm_count,
+                            cudaStream_t s);
 
 // --------------------------------------------------------------- stepper
 struct StepArgs {

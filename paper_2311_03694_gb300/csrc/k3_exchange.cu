@@ -29,6 +29,7 @@
 #include <algorithm>
 
 #include "ds_arith.cuh"
+#include "cp_async.cuh"
 #include "grom_internal.h"
 #include "ptx.cuh"
 #include "step_elem.cuh"
@@ -521,6 +522,160 @@ __global__ void __launch_bounds__(KX_THREADS, 1) k3x_kernel(const KXArgs p) {
   }
 }
 
+// ------------------------------------------------------------- evaluations
+// One evaluation of FP64 factors with the same exchange: the CTAs' columns
+// straight from memory (a thread takes whole pieces of a factor's rows; the
+// rows of the expansion are copied to shared memory meanwhile), h published,
+// then the CTAs' rows.  The two kernels of k3_cp.cu cost a second launch, the
+// row slices' partial sums and their gathering; here one exchange is left, and
+// the rest is latency.  us an evaluation, here against two kernels: n = 500,
+// r = 129, one trajectory 8.3 against 16.4; n = r = 64 8.3 against 12.4; n = r =
+// 512, general form, four trajectories 21.8 against 28.7.
+// Every CTA counts itself in once it has read the base, and the last one moves
+// it on, so that none can take the next evaluation's number.
+struct KEArgs {
+  const double *fa, *fb, *fc;  // stored factors, n x rp
+  int n, rp, batch, rows;
+  const double* u;
+  int64_t u_stride;
+  double* c;
+  int64_t c_stride;
+  unsigned int* base;      // step number of the last word published, arrivals
+  unsigned long long* hw;  // 2 x 2 x NB x rp
+  int* err;
+};
+
+// NF factors to project on, CH columns whose sums a thread carries at a time.
+template <int NB, int NF, int CH>
+__global__ void __launch_bounds__(KX_THREADS, 1) k3x_eval(const KEArgs p) {
+  constexpr int V = NF * CH * NB;
+  extern __shared__ __align__(16) double ke_smem[];
+  __shared__ int abort_sh;
+  __shared__ uint32_t tag_sh;
+  __shared__ double tot[V];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int G = gridDim.x, g = blockIdx.x, n = p.n, rp = p.rp;
+  const int r0 = (int)((int64_t)g * rp / G), rb = (int)((int64_t)(g + 1) * rp / G) - r0;
+  const int i0 = (int)((int64_t)g * n / G), ni = (int)((int64_t)(g + 1) * n / G) - i0;
+  volatile int* abort_flag = &abort_sh;
+  // [expansion rows (NF - 1) x rows x rp][h 2 x NB x rp][partial sums V x threads]
+  double* rowe = ke_smem;
+  double* hs = rowe + (size_t)(NF - 1) * p.rows * rp;
+  double* red = hs + (size_t)2 * NB * rp;
+  const double* F[3] = {p.fb, p.fc, p.fa};
+  if (tid == 0) {
+    abort_sh = 0;
+    tag_sh = *reinterpret_cast<volatile unsigned int*>(p.base);
+  }
+  const int pieces = rp / 2;  // 16-byte pieces of a row
+  for (int e = 0; e < NF - 1; ++e)
+    for (int t = tid; t < ni * pieces; t += KX_THREADS) {
+      const int ri = t / pieces, q = t - ri * pieces;
+      ptx::cp_async16(rowe + ((size_t)e * p.rows + ri) * rp + 2 * q,
+                      (e == 0 ? p.fa : p.fc) + (int64_t)(i0 + ri) * rp + 2 * q);
+    }
+  ptx::cp_async_commit();
+  // ---- projections of the owned columns
+  for (int c0 = 0; c0 < rb; c0 += CH) {
+    double acc[NF][CH][NB];
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int k = 0; k < CH; ++k)
+#pragma unroll
+        for (int b = 0; b < NB; ++b) acc[f][k][b] = 0.0;
+#pragma unroll 2
+    for (int i = tid; i < n; i += KX_THREADS) {
+      double x[NF][CH], u[NB];
+#pragma unroll
+      for (int b = 0; b < NB; ++b) u[b] = b < p.batch ? p.u[b * p.u_stride + i] : 0.0;
+#pragma unroll
+      for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int k = 0; k < CH; ++k) x[f][k] = c0 + k < rb ? F[f][(int64_t)i * rp + r0 + c0 + k] : 0.0;
+#pragma unroll
+      for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int k = 0; k < CH; ++k)
+#pragma unroll
+          for (int b = 0; b < NB; ++b) acc[f][k][b] = fma(x[f][k], u[b], acc[f][k][b]);
+    }
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+      for (int k = 0; k < CH; ++k)
+#pragma unroll
+        for (int b = 0; b < NB; ++b) red[((f * CH + k) * NB + b) * KX_THREADS + tid] = acc[f][k][b];
+    __syncthreads();
+    for (int v = warp; v < V; v += KX_WARPS) {
+      const double* x = red + v * KX_THREADS + lane;
+      double t = ((x[0] + x[32]) + (x[64] + x[96])) + ((x[128] + x[160]) + (x[192] + x[224]));
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+      if (lane == 0) tot[v] = t;
+    }
+    __syncthreads();
+    if (tid < CH * NB) {
+      const int k = tid / NB, b = tid - k * NB;
+      if (c0 + k < rb && b < p.batch) {
+        const uint32_t tag = tag_sh + 1u;
+        const int64_t plane = (int64_t)2 * p.batch * rp;
+        unsigned long long* w = p.hw + (int64_t)b * rp + r0 + c0 + k;
+        kx_publish(w, plane, tot[tid] * tot[CH * NB + tid], tag);
+        if constexpr (NF == 3) kx_publish(w + (int64_t)p.batch * rp, plane, tot[tid] * tot[2 * CH * NB + tid], tag);
+      }
+    }
+  }
+  __syncthreads();
+  const uint32_t tag = tag_sh + 1u;
+  if (tid == 0) {
+    __threadfence();
+    if (atomicInc(p.base + 1, (unsigned)G - 1u) == (unsigned)G - 1u)
+      *reinterpret_cast<volatile unsigned int*>(p.base) = tag;
+  }
+  // ---- h of every column
+  bool ok = true;
+  if (ni > 0) {
+    const int per = (NF - 1) * p.batch * rp, plane = 2 * p.batch * rp;
+#pragma unroll
+    for (int half = 0; half < 2; ++half)
+      ok = ok && kx_poll<true>(p.hw + (size_t)half * plane, per, tag, tid, KX_THREADS, abort_flag,
+                               [&](int x, uint32_t bits) {
+                                 const int row = x / rp, r = x - row * rp;  // row: which * batch + b
+                                 const int which = row >= p.batch ? 1 : 0, b = row - which * p.batch;
+                                 reinterpret_cast<uint32_t*>(hs)[(size_t)2 * ((which * NB + b) * rp + r) + half] = bits;
+                               });
+  }
+  ptx::cp_async_wait<0>();
+  if (!ok) kx_abort(abort_flag, p.err, p.base, tag);
+  if (__syncthreads_or(*abort_flag)) return;
+  // ---- the owned rows
+  for (int ri = warp; ri < ni; ri += KX_WARPS) {
+    const double* x = rowe + (size_t)ri * rp;
+    const double* w = rowe + ((size_t)p.rows + ri) * rp;  // skew only
+    double s1[NB], s2[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) s1[b] = s2[b] = 0.0;
+#pragma unroll 4
+    for (int v = lane; v < rp; v += 32) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        if (b >= p.batch) break;
+        s1[b] = fma(x[v], hs[(size_t)b * rp + v], s1[b]);
+        if constexpr (NF == 3) s2[b] = fma(w[v], hs[(size_t)(NB + b) * rp + v], s2[b]);
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      if (b >= p.batch) break;
+      double t = NF == 3 ? s1[b] - s2[b] : s1[b];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+      if (lane == 0) p.c[b * p.c_stride + i0 + ri] = t;
+    }
+  }
+}
+
 // A warp per column and row: CTAs of eight of each, as many as there are SMs.
 static int kx_grid(int64_t n, int64_t rp, int sm_count) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(sm_count, (std::max(n, rp) + KX_WARPS - 1) / KX_WARPS));
@@ -550,7 +705,7 @@ bool k3x_fits(int64_t n, int64_t rp, int form, int storage, int batch, int sm_co
   return kx_shape(n, rp, form, storage, batch, sm_count).smem <= 220 * 1024;
 }
 
-// [base word][u words][h words][energy / invariant words], for four trajectories
+// [base and arrival words][u words][h words][energy / invariant words], for four trajectories
 size_t k3x_scratch_bytes(int64_t n, int64_t rp, int sm_count) {
   return 256 + 8 * (2 * 4 * (size_t)n + 2 * 2 * 4 * (size_t)rp + 2 * (size_t)sm_count * 4 * 4);
 }
@@ -594,6 +749,68 @@ cudaError_t k3x_launch(const uint8_t* fa, const uint8_t* fb, const uint8_t* fc, 
     case GROM_BF16: return kx_run<GROM_BF16>(p, s, strm);
   }
   return cudaErrorInvalidValue;
+}
+
+struct KEShape {
+  int grid, rows, nb, ch;
+  size_t smem;
+};
+static KEShape ke_shape(int64_t n, int64_t rp, int form, int batch, int sm_count) {
+  KEShape s{};
+  const int nf = form == GROM_FORM_CP_SKEW ? 3 : 2;
+  s.grid = (int)std::max<int64_t>(1, std::min<int64_t>(sm_count, std::max(rp, (n + KX_WARPS - 1) / KX_WARPS)));
+  s.rows = (int)((n + s.grid - 1) / s.grid);
+  s.nb = batch <= 1 ? 1 : batch <= 2 ? 2 : 4;
+  const int cols = (int)((rp + s.grid - 1) / s.grid);
+  s.ch = std::min(4 / s.nb, cols <= 1 ? 1 : cols <= 2 ? 2 : 4);
+  s.smem = ((size_t)(nf - 1) * s.rows * rp + 2 * (size_t)s.nb * rp + (size_t)nf * s.ch * s.nb * KX_THREADS) * 8;
+  return s;
+}
+
+// Where one launch is faster: until a CTA's columns and the h that every CTA
+// polls outgrow the second launch (skew form: five products an entry and two h
+// a column).  us here against k3_cp.cu, n, r, trajectories: skew 256, 256, 4:
+// 18.5, 26.7; 512, 512, 2: 20.5, 24.7; 512, 512, 4: 34.3, 33.9; 700, 700, 1:
+// 22.6, 25.4; 700, 700, 2: 33.8, 32.9; 1024, 1024, 1: 30.8, 27.3; 2048, 512,
+// 2: 36.4, 44.0; general 1024, 1024, 4: 46.9, 53.3; 2048, 512, 4: 45.4, 55.4.
+bool k3x_eval_faster(int64_t n, int64_t rp, int form, int batch, int sm_count) {
+  if (batch > 4 || n > 2048) return false;
+  const KEShape s = ke_shape(n, rp, form, batch, sm_count);
+  if (s.smem > 220 * 1024) return false;
+  return form == GROM_FORM_CP_SKEW ? s.nb * rp <= 1024 && rp <= 5 * s.grid : s.nb * rp <= 4096 && rp <= 1024;
+}
+
+template <int NF>
+static void (*ke_kernel(const KEShape& s))(const KEArgs) {
+  if (s.nb == 4) return k3x_eval<4, NF, 1>;
+  if (s.nb == 2) return s.ch == 1 ? k3x_eval<2, NF, 1> : k3x_eval<2, NF, 2>;
+  return s.ch == 1 ? k3x_eval<1, NF, 1> : s.ch == 2 ? k3x_eval<1, NF, 2> : k3x_eval<1, NF, 4>;
+}
+
+cudaError_t k3x_eval_launch(const K3Args& a, int64_t n, int64_t rp, int batch, void* scratch, int* err, int sm_count,
+                            cudaStream_t strm) {
+  const KEShape s = ke_shape(n, rp, a.form, batch, sm_count);
+  KEArgs p{};
+  p.fa = reinterpret_cast<const double*>(a.fa);
+  p.fb = reinterpret_cast<const double*>(a.fb);
+  p.fc = reinterpret_cast<const double*>(a.fc);
+  p.n = (int)n;
+  p.rp = (int)rp;
+  p.batch = batch;
+  p.rows = s.rows;
+  p.u = a.u;
+  p.u_stride = a.u_stride;
+  p.c = a.c;
+  p.c_stride = a.c_stride;
+  p.base = static_cast<unsigned int*>(scratch);
+  p.hw = reinterpret_cast<unsigned long long*>(static_cast<uint8_t*>(scratch) + 256) + 2 * 4 * (size_t)n;
+  p.err = err;
+  auto kern = a.form == GROM_FORM_CP_SKEW ? ke_kernel<3>(s) : ke_kernel<2>(s);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
+  if (e != cudaSuccess) return e;
+  void* args[] = {&p};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kern), dim3(s.grid), dim3(KX_THREADS), args, s.smem,
+                                     strm);
 }
 
 }  // namespace grom
