@@ -115,19 +115,30 @@ __global__ void k_als_norm(const double* __restrict__ src, int64_t total, double
   if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
+// The tile (row tj <= column ti) at place x of a triangle taken row by row.
+__device__ __forceinline__ void triangle_tile(int64_t x, int64_t& ti, int64_t& tj) {
+  ti = (int64_t)((sqrt((double)(8 * x + 1)) - 1.0) / 2.0);
+  while ((ti + 1) * (ti + 2) / 2 <= x) ++ti;
+  while (ti * (ti + 1) / 2 > x) --ti;
+  tj = x - ti * (ti + 1) / 2;
+}
+
 // G = F^T F for F (n x r, row-major FP64), 16 x 16 output tiles; G is
 // symmetric, so only the tiles on and above the diagonal are computed (FP64
 // runs at about two operations per clock per SM here) and mirrored.  Chunks
 // of 64 rows with the next one in flight, so that two warps per FP64 pipe
-// keep it busy (n = 512, r = 256: 68.4 us against 75.8 with chunks of
-// 16; the pipe's own time is 32 us).
+// keep it busy.  A CTA per tile of the triangle and none beside it: in a
+// square grid the CTAs that leave at once take places of the first wave, and
+// the working ones pair up on SMs while others idle (n = 512, r = 256, 136
+// tiles: 37.9 us against 68.0; the pipe's own time is 32 us).
 constexpr int GR_K = 64;
 __global__ void __launch_bounds__(256) k_gram(const double* __restrict__ F, int64_t n, int64_t r,
                                               double* __restrict__ G) {
-  if (blockIdx.x < blockIdx.y) return;  // whole block, before any barrier
   __shared__ double a[GR_K][17], b[GR_K][17];
+  int64_t ti, tj;
+  triangle_tile(blockIdx.x, ti, tj);
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int64_t ra = (int64_t)blockIdx.y * 16 + tx, col = (int64_t)blockIdx.x * 16 + tx;
+  const int64_t ra = tj * 16 + tx, col = ti * 16 + tx;
   double na[GR_K / 16], nb[GR_K / 16];
   auto fetch = [&](int64_t i0) {
 #pragma unroll
@@ -151,7 +162,7 @@ __global__ void __launch_bounds__(256) k_gram(const double* __restrict__ F, int6
     for (int q = 0; q < GR_K; ++q) s = fma(a[q][ty], b[q][tx], s);
     __syncthreads();
   }
-  const int64_t row = (int64_t)blockIdx.y * 16 + ty;
+  const int64_t row = tj * 16 + ty;
   if (row < r && col < r) {
     G[row * r + col] = s;
     G[col * r + row] = s;
@@ -187,56 +198,89 @@ constexpr int UT = 16;  // trailing-update tile
 // steps for the reciprocal square root, y <- y (3 - m y^2) / 2, bring to FP64
 // precision (each step about doubles the correct bits).  FP64 division and
 // square root cost thousands of cycles on this part, a step of this a few
-// hundred.
+// hundred.  The exponents are moved as integers: only the steps' six FP64
+// operations are left on the chain.
 __device__ __forceinline__ double rsqrt_nr(double d) {
-  const int e = ilogb(d) >> 1;
-  const double m = scalbn(d, -2 * e);
-  double y = (double)rsqrtf((float)m);
-  y = y * (1.5 - 0.5 * m * y * y);
-  y = y * (1.5 - 0.5 * m * y * y);
-  return scalbn(y, -e);
+  int hi = __double2hiint(d), up = 0;
+  int lo = __double2loint(d);
+  if (hi < 0x00100000) {  // subnormal: 2^108 d first
+    d *= 0x1p108;
+    hi = __double2hiint(d);
+    lo = __double2loint(d);
+    up = 54;
+  }
+  const int e = ((hi >> 20) - 1023) >> 1;
+  hi -= e * (1 << 21);
+  const double h = __hiloint2double(hi - (1 << 20), lo);  // m / 2
+  double y = f2d_int(rsqrtf(d2f_int(__hiloint2double(hi, lo))));
+  y = y * (1.5 - h * y * y);
+  y = y * (1.5 - h * y * y);
+  return __hiloint2double(__double2hiint(y) - (e - up) * (1 << 20), __double2loint(y));
 }
 
 // Factors the diagonal block at (kb, kb) in place (lower), right-looking, and
 // stores the reciprocals of its pivots in rdiag[kb ..].  A pivot that is not
-// positive and finite sets *flag.  One CTA of four warps, one per FP64 pipe:
-// lane = column, warp w holds rows w, w + 4, ... in registers, every warp
-// forms the pivot's reciprocal root itself, and the next column goes through
-// shared memory: one barrier a pivot, where a thread per entry took three.
-// The chain of some ten dependent FP64 operations a pivot is what bounds it:
-// 38.2 us a block against 50.5.
+// positive and finite sets *flag.  The chain of dependent FP64 operations from
+// one pivot to the next bounds it (some 70 cycles each), so warp 0, alone on
+// its FP64 pipe, runs only that chain: lane = row, it holds column c, takes
+// the pivot's reciprocal root, scales the column and brings column c + 1 up to
+// date.  Warps 1 to 3 hold the block (lane = column, rows warp - 1, + 3, ...)
+// and apply column c - 1 meanwhile; what warp 0 gets of column c + 1 is
+// therefore short of the columns c - 1 and c, which it applies itself.  Every
+// entry sees the columns in the same order as one after the other.  One
+// barrier a pivot; us a block, 32 pivots: 24.6 against 38.2 with the update
+// between two pivots, 50.5 with a thread per entry.
+constexpr int CD_ROWS = (CH + 2) / 3;
 __global__ void __launch_bounds__(128) k_chol_diag(double* H, int64_t r, int64_t kb, double* rdiag, int* flag) {
-  __shared__ double Ls[CH][CH + 1], col[2][CH];
+  __shared__ double Ls[CH][CH + 1], col[2][CH], lb[2][CH];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nb = (int)(r - kb < CH ? r - kb : CH);
-  double a[CH / 4];
+  auto entry = [&](int i, int j) {
+    return i < nb && j <= i ? H[(kb + i) * r + kb + j] : (j == i ? 1.0 : 0.0);
+  };
+  double a[CD_ROWS];
+  double cc = 0.0, lp = 0.0;  // warp 0: column c, the scaled column c - 1
+  if (w == 0) {
+    cc = entry(lane, 0);
+  } else {
 #pragma unroll
-  for (int k = 0; k < CH / 4; ++k) {
-    const int i = w + 4 * k;
-    a[k] = i < nb && lane <= i ? H[(kb + i) * r + kb + lane] : (lane == i ? 1.0 : 0.0);
-    if (lane == 0) col[0][i] = a[k];
+    for (int k = 0; k < CD_ROWS; ++k) {
+      const int i = w - 1 + 3 * k;
+      a[k] = i < CH ? entry(i, lane) : 0.0;
+      if (i < CH && lane == 1) col[1][i] = a[k];
+    }
   }
   __syncthreads();
   for (int c = 0; c < nb; ++c) {
-    const double* cc = col[c & 1];  // column c, rows >= c
-    const double d = cc[c];
-    if (!(d > 0.0) || !isfinite(d)) {  // the same value in every thread
-      if (threadIdx.x == 0) atomicExch(flag, 1);
-      return;
-    }
-    const double y = rsqrt_nr(d);
-    const double l = cc[lane] * y;  // L[lane][c] for lane > c
-    if (w == 0) Ls[lane][c] = lane > c ? l : lane == c ? d * y : 0.0;
-    if (w == 1 && lane == 0) rdiag[kb + c] = y;
+    int bad = 0;
+    if (w == 0) {
+      const double d = __shfl_sync(0xffffffffu, cc, c);
+      const long long bits = __double_as_longlong(d);
+      if (bits <= 0 || bits >= 0x7ff0000000000000ll) {  // not positive and finite; the same in every lane
+        if (lane == 0) atomicExch(flag, 1);
+        bad = 1;
+      } else {
+        double x = col[(c + 1) & 1][lane];
+        if (c > 0) x = fma(-__shfl_sync(0xffffffffu, lp, (c + 1) & 31), lp, x);
+        const double y = rsqrt_nr(d);
+        const double l = cc * y;  // L[lane][c] for lane > c
+        Ls[lane][c] = lane > c ? l : lane == c ? d * y : 0.0;
+        lb[c & 1][lane] = l;
+        if (lane == 0) rdiag[kb + c] = y;
+        cc = fma(-__shfl_sync(0xffffffffu, l, (c + 1) & 31), l, x);
+        lp = l;
+      }
+    } else {
+      const double l = c > 0 ? lb[(c - 1) & 1][lane] : 0.0;
 #pragma unroll
-    for (int k = 0; k < CH / 4; ++k) {
-      const int i = w + 4 * k;
-      const double li = __shfl_sync(0xffffffffu, l, i);
-      if (i <= c) continue;  // warp-uniform
-      a[k] = fma(-li, l, a[k]);
-      if (lane == c + 1) col[(c + 1) & 1][i] = a[k];
+      for (int k = 0; k < CD_ROWS; ++k) {
+        const int i = w - 1 + 3 * k;
+        if (i < c || i >= CH) continue;  // warp-uniform
+        if (c > 0) a[k] = fma(-__shfl_sync(0xffffffffu, l, i), l, a[k]);
+        if (lane == c + 2) col[c & 1][i] = a[k];
+      }
     }
-    __syncthreads();
+    if (__syncthreads_or(bad)) return;
   }
   for (int x = threadIdx.x; x < nb * CH; x += 128)
     if (x % CH < nb) H[(kb + x / CH) * r + kb + x % CH] = Ls[x / CH][x % CH];
@@ -265,11 +309,8 @@ __global__ void k_chol_panel(double* H, int64_t r, int64_t kb, const double* __r
 // (one thread per entry) per UT x UT tile of the lower trailing matrix.
 __global__ void __launch_bounds__(UT * UT) k_chol_update(double* H, int64_t r, int64_t kb) {
   __shared__ double Pi[UT][CH + 1], Pj[UT][CH + 1];
-  const int64_t x = blockIdx.x;
-  int64_t ti = (int64_t)((sqrt((double)(8 * x + 1)) - 1.0) / 2.0);
-  while ((ti + 1) * (ti + 2) / 2 <= x) ++ti;
-  while (ti * (ti + 1) / 2 > x) --ti;
-  const int64_t tj = x - ti * (ti + 1) / 2;
+  int64_t ti, tj;
+  triangle_tile(blockIdx.x, ti, tj);
   const int64_t i0 = kb + CH + ti * UT, j0 = kb + CH + tj * UT;
   const int tx = threadIdx.x % UT, ty = threadIdx.x / UT;
   for (int e = threadIdx.x; e < UT * CH; e += UT * UT) {
@@ -298,11 +339,12 @@ __global__ void k_transpose(const double* __restrict__ L, int64_t r, double* __r
 // L z = m_i, backward L^T a_i = z, 32 unknowns at a time, SV_ROWS rows per CTA
 // and four warps per row.  Per block the solved unknowns' contribution is
 // summed with lanes over the contracted index (coalesced rows of L or L^T,
-// eight unknowns a warp, a butterfly across the lanes), then the row's first
-// warp (the rows of a CTA run at their own pace) solves the 32 x 32 triangle, staged in shared memory with the
+// eight unknowns a warp, a butterfly across the lanes), then one warp of the
+// row (each row's on another FP64 pipe; the rows of a CTA run at their own
+// pace) solves the 32 x 32 triangle, staged in shared memory with the
 // reciprocals of its pivots, with shuffles.
 // n r^2 multiply-adds (53 us of the FP64 pipe at n = 512, r = 256) and the
-// triangles' chains of 2 r shuffle-multiply-add steps bound it: 221 us
+// triangles' chains of 2 r shuffle-multiply-add steps bound it: 192 us
 // there; one warp per row, with 32 sums of its own, took 400.
 constexpr int SV_ROWS = 4, SV_WARPS = 4, SV_T = CH / SV_WARPS;
 
@@ -366,7 +408,7 @@ __global__ void __launch_bounds__(32 * SV_ROWS * SV_WARPS)
       const double v8 = warp_sum8(acc, lane);
       if ((lane & 3) == 0 && sub * SV_T + (lane >> 2) < nb) y[a0 + sub * SV_T + (lane >> 2)] -= v8;
       row_sync();
-      if (sub == 0) {
+      if (sub == row % SV_WARPS) {
         double v = lane < nb ? y[a0 + lane] : 0.0;
         for (int k = 0; k < nb; ++k) {
           const int c = pass ? nb - 1 - k : k;
@@ -507,8 +549,8 @@ grom_status als_grow(grom_als* s, int64_t r) {
 
 // Gram matrix of factor q (on the device).
 grom_status gram_of(grom_als* s, int q, int64_t r) {
-  dim3 grid((unsigned)((r + 15) / 16), (unsigned)((r + 15) / 16));
-  k_gram<<<grid, dim3(16, 16), 0, s->stream>>>(s->f[q], s->n, r, s->gram[q]);
+  const int64_t t = (r + 15) / 16;
+  k_gram<<<(unsigned)(t * (t + 1) / 2), dim3(16, 16), 0, s->stream>>>(s->f[q], s->n, r, s->gram[q]);
   GROM_CUDA_TRY(cudaGetLastError());
   return GROM_OK;
 }
