@@ -344,9 +344,11 @@ __global__ void k_transpose(const double* __restrict__ L, int64_t r, double* __r
 // pace) solves the 32 x 32 triangle, staged in shared memory with the
 // reciprocals of its pivots, with shuffles.
 // n r^2 multiply-adds (53 us of the FP64 pipe at n = 512, r = 256) and the
-// triangles' chains of 2 r shuffle-multiply-add steps bound it: 192 us
-// there; one warp per row, with 32 sums of its own, took 400.
+// triangles' chains of 2 r shuffle-multiply-add steps bound it: 154 us
+// there (192 with the triangle loaded when its turn comes); one warp per row,
+// with 32 sums of its own, took 400.
 constexpr int SV_ROWS = 4, SV_WARPS = 4, SV_T = CH / SV_WARPS;
+constexpr int SV_FETCH = (CH * CH + 32 * (SV_WARPS - 1) - 1) / (32 * (SV_WARPS - 1));
 
 // Butterfly sums over the 32 lanes of v[0 .. 8): every pair of partial sums
 // is added in the order 16, 8, 4, 2, 1, and lane l ends with v[(l >> 2) & 7]
@@ -375,7 +377,6 @@ __global__ void __launch_bounds__(32 * SV_ROWS * SV_WARPS)
   __shared__ double Bs[SV_ROWS][CH][CH + 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, row = w / SV_WARPS, sub = w % SV_WARPS;
   const int64_t i0 = (int64_t)blockIdx.x * SV_ROWS, i = i0 + row;
-  const int rt = threadIdx.x % (32 * SV_WARPS);  // thread of the row's four warps
   double* y = ybuf + (size_t)row * r;
   double(*B)[CH + 1] = Bs[row];
   auto row_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(row + 1), "r"(32 * SV_WARPS) : "memory"); };
@@ -385,15 +386,34 @@ __global__ void __launch_bounds__(32 * SV_ROWS * SV_WARPS)
   }
   __syncthreads();
   const int64_t last = (r - 1) / CH * CH;
+  // the triangle of the next block, on its way while the row's solver works:
+  // by the row's other warps, in their registers
+  const int solver = row % SV_WARPS;
+  const int ft = (sub + SV_WARPS - 1 - solver) % SV_WARPS * 32 + lane;  // 0 .. 95 in them
+  double bn[SV_FETCH], rn = 0.0;
+  auto fetch = [&](const double* M, int64_t a0, int nb) {
+#pragma unroll
+    for (int k = 0; k < SV_FETCH; ++k) {
+      const int t = ft + k * 32 * (SV_WARPS - 1);
+      bn[k] = t < CH * CH && t / CH < nb && t % CH < nb ? M[(a0 + t / CH) * r + a0 + t % CH] : 0.0;
+    }
+    if (ft < nb) rn = rdiag[a0 + ft];
+  };
+  if (sub != solver) fetch(L, 0, (int)(r < CH ? r : CH));
   for (int pass = 0; pass < 2; ++pass) {
     const double* M = pass ? Lt : L;
     for (int64_t x = 0; x <= last; x += CH) {
       const int64_t a0 = pass ? last - x : x;
       const int nb = (int)(r - a0 < CH ? r - a0 : CH);
       const int64_t q0 = pass ? a0 + nb : 0, q1 = pass ? r : a0;  // the solved unknowns
-      for (int t = rt; t < CH * CH; t += 32 * SV_WARPS)
-        if (t / CH < nb && t % CH < nb) B[t / CH][t % CH] = M[(a0 + t / CH) * r + a0 + t % CH];
-      if (rt < nb) B[rt][CH] = rdiag[a0 + rt];
+      if (sub != solver) {
+#pragma unroll
+        for (int k = 0; k < SV_FETCH; ++k) {
+          const int t = ft + k * 32 * (SV_WARPS - 1);
+          if (t < CH * CH) B[t / CH][t % CH] = bn[k];
+        }
+        if (ft < CH) B[ft][CH] = rn;
+      }
       double acc[SV_T];
 #pragma unroll
       for (int t = 0; t < SV_T; ++t) acc[t] = 0.0;
@@ -408,7 +428,7 @@ __global__ void __launch_bounds__(32 * SV_ROWS * SV_WARPS)
       const double v8 = warp_sum8(acc, lane);
       if ((lane & 3) == 0 && sub * SV_T + (lane >> 2) < nb) y[a0 + sub * SV_T + (lane >> 2)] -= v8;
       row_sync();
-      if (sub == row % SV_WARPS) {
+      if (sub == solver) {
         double v = lane < nb ? y[a0 + lane] : 0.0;
         for (int k = 0; k < nb; ++k) {
           const int c = pass ? nb - 1 - k : k;
@@ -423,6 +443,9 @@ __global__ void __launch_bounds__(32 * SV_ROWS * SV_WARPS)
           y[a0 + lane] = v;
           if (pass && i < n) A[i * r + a0 + lane] = v;
         }
+      } else if (x < last || pass == 0) {
+        const int64_t a1 = pass ? a0 - CH : x < last ? a0 + CH : last;
+        fetch(x < last ? M : Lt, a1, (int)(r - a1 < CH ? r - a1 : CH));
       }
       row_sync();
     }
