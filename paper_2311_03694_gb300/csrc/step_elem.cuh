@@ -29,9 +29,15 @@ __device__ __forceinline__ double step_ext(int k, const double (&g)[3]) {
 // onto the extrapolation, six FP64 operations at order 3.
 __device__ __forceinline__ double step_plain_elem(const double (&bdt)[3], int k, const double (&u)[3],
                                                   const double (&g)[3], double hd) {
-  double y = step_ext(k, g);
-  if (k == 3) y = fma(bdt[2], u[2], y);
-  if (k >= 2) y = fma(bdt[1], u[1], y);
+  double y;
+  if (k == 3) {  // uniform: no predicated-off FP64 instruction on the usual way
+    y = fma(3.0, __dsub_rn(g[0], g[1]), g[2]);
+    y = fma(bdt[2], u[2], y);
+    y = fma(bdt[1], u[1], y);
+  } else {
+    y = step_ext(k, g);
+    if (k == 2) y = fma(bdt[1], u[1], y);
+  }
   y = fma(bdt[0], u[0], y);
   return __dmul_rn(-y, hd);
 }
@@ -62,7 +68,7 @@ __device__ __forceinline__ double step_elem(const StepArgs& a, double* h, int64_
   double u[3] = {0.0, 0.0, 0.0}, g[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    if (q < k) {
+    if (PLAIN || q < k) {  // plain: all six loads in flight at once, a lower order leaves some unused
       const int m = m0 - q < 0 ? m0 - q + 3 : m0 - q;
       u[q] = h[m * n + i];
       g[q] = q == 0 ? nl : h[(3 + m) * n + i];
