@@ -300,9 +300,19 @@ static bool use_k3o(const grom_rom* r, int batch) {
   return r->kernel_choice == GROM_KERNEL_AUTO && k3o_faster(r->n, r->rank, batch, r->form == GROM_FORM_CP_SKEW);
 }
 
+// A cooperative launch needs all its CTAs on the device at once; a context that
+// may use fewer SMs than the device has is refused it.  The caller then takes
+// the next path.
+static bool not_placed(cudaError_t e) {
+  if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return false;
+  cudaGetLastError();
+  return true;
+}
+
 // Evaluations of a few trajectories of FP64 factors in one launch
-// (k3_exchange.cu) in place of K3's two.  FP32 and BF16 factors keep K3: their
-// FP32 sums would be taken in another order.
+// (k3_exchange.cu) in place of K3's two, which serve where it cannot be
+// placed.  FP32 and BF16 factors keep K3: their FP32 sums would be taken in
+// another order.
 static bool use_k3x_eval(const grom_rom* r, int batch) {
   return is_cp(r) && r->storage == GROM_F64 && r->kernel_choice == GROM_KERNEL_AUTO &&
          k3x_eval_faster(r->n, r->k3.rb, r->form, batch, r->sm_count);
@@ -479,6 +489,15 @@ static K1TArgs k1t_args(const grom_rom* r, const grom_traj* t) {
     a.active = t->active;
   }
   return a;
+}
+
+// Evaluations of the CP forms outside the batched GEMMs.
+static cudaError_t k3_few_launch(grom_rom* r, const K3Args& a, int batch) {
+  if (use_k3x_eval(r, batch)) {
+    const cudaError_t e = k3x_eval_launch(a, r->n, r->k3.rb, batch, r->k3x_scratch, r->err, r->sm_count, r->stream);
+    if (!not_placed(e)) return e;
+  }
+  return k3_launch(r->k3, r->storage, a, batch, r->stream);
 }
 
 static K3Args k3_args(grom_rom* r) {
@@ -985,8 +1004,7 @@ grom_status grom_nonlinear(grom_rom* r, int32_t batch, const double* u, double* 
         : use_k3d(r, batch) ? k3d_launch(r->k3, a, r->k3d_factors, batch, r->max_batch, r->k3d_scratch, r->sm_count,
                                          r->stream)
         : use_k3g(r, batch) ? k3g_launch(r->k3, r->storage, a, batch, r->max_batch, r->k3g_scratch, r->sm_count, r->stream)
-        : use_k3x_eval(r, batch) ? k3x_eval_launch(a, r->n, r->k3.rb, batch, r->k3x_scratch, r->err, r->sm_count, r->stream)
-                            : k3_launch(r->k3, r->storage, a, batch, r->stream);
+                            : k3_few_launch(r, a, batch);
     if (e1) prof_record(e1, r->stream);
   }
   if (e != cudaSuccess) return cuda_fail(e, "grom_nonlinear launch");
@@ -1288,7 +1306,8 @@ grom_status grom_step(grom_traj* t, int32_t nsteps, double* energy, double* inva
   if (!full_ready(r)) return fail(GROM_ERR_INVALID_ARG, "grom_step: tensor rows missing");
   // CP forms with a few trajectories: all steps in one persistent launch,
   // without grid barriers where the factors fit shared memory by columns and
-  // by rows
+  // by rows (the next of the two, then the kernels below, where the launch
+  // cannot be placed)
   if (r->diagonal && is_cp(r) && !t->active && !r->prof && nsteps >= 4 && !use_k3t(r, t->batch, false)) {
     const uint8_t *fa = r->op, *fb = r->op + r->panel_bytes, *fc = r->op + 2 * r->panel_bytes;
     const bool few = t->batch <= k3p_max_batch(r->storage);
@@ -1297,11 +1316,11 @@ grom_status grom_step(grom_traj* t, int32_t nsteps, double* energy, double* inva
     if (few && k3x_fits(r->n, r->k3.rb, r->form, r->storage, t->batch, r->sm_count))
       e = k3x_launch(fa, fb, fc, r->form, r->n, r->k3.rb, r->storage, t->batch, nsteps, a, r->k3x_scratch, r->sm_count,
                      r->stream);
-    else if (few && k3p_fits(r->n, r->k3.rb, r->storage, t->batch, r->sm_count))
+    if (not_placed(e) && few && k3p_fits(r->n, r->k3.rb, r->storage, t->batch, r->sm_count))
       e = k3p_launch(fa, fb, fc, r->form, r->n, r->k3.rb, r->storage, t->batch, nsteps, a, r->k3p_scratch, r->sm_count,
                      r->stream);
     if (e == cudaSuccess) return GROM_OK;
-    if (e != cudaErrorNotSupported) return cuda_fail(e, "grom_step persistent launch");
+    if (!not_placed(e)) return cuda_fail(e, "grom_step persistent launch");
   }
   // full G-ROM with the skew-packed tensor and a few trajectories: all steps
   // in one persistent launch (falls back to the graphs below when the launch
