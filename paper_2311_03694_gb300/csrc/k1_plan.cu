@@ -90,10 +90,6 @@ K1Plan k1_plan(int64_t n, int storage, int sm_count, int packed, int64_t m) {
   if (grid > p.T) grid = p.T;
   if (grid < 1) grid = 1;
   p.grid = (int)grid;
-  // one chunk a test index and a CTA for each: no second launch for the sums
-  // over CTAs (n = 64 F64, an evaluation through the
-  // binding: 6.2 us against 10.2)
-  p.whole = !packed && p.cpi == 1 && grid == n;
   const int64_t per = (p.T + grid - 1) / grid;
   p.maxseg = (int)((per + p.cpi - 1) / p.cpi + 1);
   const int64_t per_traj = k1_traj_smem(p, storage);

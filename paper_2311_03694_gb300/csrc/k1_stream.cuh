@@ -20,6 +20,8 @@
 // (deterministic, no atomics).
 #pragma once
 
+#include <functional>
+
 #include "ds_arith.cuh"
 #include "grom_internal.h"
 #include "ptx.cuh"
@@ -151,7 +153,10 @@ __device__ __forceinline__ void k1_load_state(const K1Plan& pl, const K1Args& a,
   }
 }
 
-template <int ST, int QM, int NB>
+// WHOLE (k1_whole): the CTA's one test index is finalised here.  A template
+// parameter, not a field of the plan: tested at run time it took 5 to 9
+// registers of every instance.
+template <int ST, int QM, int NB, bool WHOLE>
 __global__ void __launch_bounds__(K1_THREADS, 1) k1_stream_kernel(const K1Plan pl, const K1Args a, const int b0) {
   using TR = K1Traits<ST>;
   extern __shared__ uint8_t smem_raw[];
@@ -162,7 +167,7 @@ __global__ void __launch_bounds__(K1_THREADS, 1) k1_stream_kernel(const K1Plan p
   volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + K1_STAGES);
   uint8_t* ureg = reinterpret_cast<uint8_t*>(empty + K1_STAGES) + 16;
 
-  __shared__ double wsum[K1_CONSUMERS / 32][NB];  // pl.whole: the warps' sums of the CTA's test index
+  __shared__ double wsum[WHOLE ? K1_CONSUMERS / 32 : 1][NB];  // the warps' sums of the CTA's test index
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t n = pl.n, np = pl.np, row_bytes = pl.row_bytes;
   const int64_t G = gridDim.x;
@@ -272,12 +277,10 @@ __global__ void __launch_bounds__(K1_THREADS, 1) k1_stream_kernel(const K1Plan p
       }
       if (lane == 0) {
         const int64_t seg = i_seg - first_i;
-        double* dst = a.part + (((int64_t)blockIdx.x * pl.maxseg + seg) * (K1_CONSUMERS / 32) + warp) * NB;
+        double* dst = WHOLE ? wsum[warp]
+                            : a.part + (((int64_t)blockIdx.x * pl.maxseg + seg) * (K1_CONSUMERS / 32) + warp) * NB;
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-          dst[b] = contrib[b];
-          if (pl.whole) wsum[warp][b] = contrib[b];
-        }
+        for (int b = 0; b < NB; ++b) dst[b] = contrib[b];
       }
     };
 
@@ -436,7 +439,7 @@ __global__ void __launch_bounds__(K1_THREADS, 1) k1_stream_kernel(const K1Plan p
       }
     }
     if (cur_i >= 0 && !__any_sync(0xffffffffu, *abort_flag != 0)) flush(cur_i);
-    if (pl.whole && !a.skip_finalize) {
+    if constexpr (WHOLE) {
       ptx::named_sync(1, K1_CONSUMERS);
       if (tid < a.nb && !*abort_flag) {
         const int bg = b0 + tid;
@@ -478,9 +481,19 @@ __global__ void k1_finalize_kernel(const K1Plan pl, const K1Args a, const int b0
   dst[i] = s;
 }
 
+// Whether the rows of u and c of this pass share memory.
+inline bool k1_shared_rows(const K1Plan& pl, const K1Args& a, int b0) {
+  if (a.taken) return false;
+  const double *u0 = a.u + b0 * a.u_stride, *u1 = u0 + (a.nb - 1) * a.u_stride + pl.n;
+  const double *c0 = a.c + b0 * a.c_stride, *c1 = c0 + (a.nb - 1) * a.c_stride + pl.n;
+  return std::less<const double*>()(u0, c1) && std::less<const double*>()(c0, u1);
+}
+
 template <int ST, int QM, int NB>
 cudaError_t k1_launch_one(const K1Plan& pl, const K1Args& a, int b0, cudaStream_t s) {
-  auto kern = k1_stream_kernel<ST, QM, NB>;
+  // not where c may be u: a CTA writes its c while others still read u
+  const bool whole = QM == 1 && k1_whole(pl) && !a.skip_finalize && !k1_shared_rows(pl, a, b0);
+  auto kern = whole ? k1_stream_kernel<ST, QM, NB, QM == 1> : k1_stream_kernel<ST, QM, NB, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
   if (e != cudaSuccess) return e;
   if (a.ev0) prof_record(a.ev0, s);
@@ -488,7 +501,7 @@ cudaError_t k1_launch_one(const K1Plan& pl, const K1Args& a, int b0, cudaStream_
   e = cudaGetLastError();
   if (e == cudaSuccess && a.ev1) e = prof_record(a.ev1, s);
   if (e != cudaSuccess) return e;
-  if (a.skip_finalize || pl.whole) return cudaSuccess;
+  if (a.skip_finalize || whole) return cudaSuccess;
   const int64_t total = pl.n * a.nb;
   k1_finalize_kernel<NB><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(pl, a, b0);
   return cudaGetLastError();

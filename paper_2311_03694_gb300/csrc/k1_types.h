@@ -31,7 +31,6 @@ struct K1Plan {
   int64_t T;           // total chunks = n * cpi
   int grid;            // persistent CTAs
   int maxseg;          // max test-index segments per CTA
-  int whole;           // 1: every CTA covers one whole test index and finalises it itself (dense layout)
   int qm;              // vector positions per consumer thread per row (1,2,4,8)
   int nb_max;          // trajectories per pass
   size_t smem;         // dynamic shared memory
@@ -42,6 +41,11 @@ struct K1Plan {
   int64_t lp;          // stored elements per row: round_up(max(h, 1), 64)
   int64_t lw;          // transposed-term window per CTA: maxseg - 1 + lp
 };
+// Dense layout, one chunk a test index and a CTA for each: a CTA can write its c
+// itself, with no second launch for the sums over CTAs (n = 64 F64, an
+// evaluation through the binding: 6.2 us against 10.2).  Such rows are at most
+// 256 vectors wide (QM = 1).
+inline bool k1_whole(const K1Plan& p) { return !p.packed && p.cpi == 1 && p.grid == p.n; }
 // Rows between a consumer thread's consecutive rows of a chunk: the row
 // groups of the packed layout, else the rows that share the consumer threads
 // (the kernels derive the same value; kept out of K1Plan, whose size is part

@@ -205,8 +205,40 @@ static void refused_launches() {
   grom_destroy(rom);
 }
 
+// A dense full ROM with a CTA per test index: one kernel an evaluation, two
+// where c is u (a CTA of the one-kernel form writes c while others read u).
+static void whole_test_indices() {
+  for (int storage : {GROM_F64, GROM_F32X2, GROM_F32, GROM_BF16}) {
+    const int n = 64;
+    std::vector<double> C((size_t)n * n * n, 0.125), a(n, 1.0), u(8 * n, 0.5), c(8 * n);
+    grom_desc d{};
+    d.n = n;
+    d.form = GROM_FORM_FULL;
+    d.storage = storage;
+    d.tensor = C.data();
+    d.stiffness_diag = a.data();
+    d.nu = 1e-2;
+    d.dt = 1e-3;
+    d.order = 3;
+    d.max_batch = 8;
+    grom_rom* rom = nullptr;
+    check(grom_create(&d, nullptr, &rom) == GROM_OK, "create");
+    for (int batch : {1, 8}) {
+      g_launched.clear();
+      check(grom_nonlinear(rom, batch, u.data(), c.data()) == GROM_OK, "evaluation");
+      const size_t apart = g_launched.size();
+      check(!ran("k1_finalize"), "no second kernel");
+      g_launched.clear();
+      check(grom_nonlinear(rom, batch, u.data(), u.data()) == GROM_OK, "evaluation in place");
+      check(ran("k1_finalize") && g_launched.size() == 2 * apart, "the sums in a second kernel where c is u");
+    }
+    grom_destroy(rom);
+  }
+}
+
 int main() {
   refused_launches();
+  whole_test_indices();
   std::printf("%ld checks, %ld failed\n", checks, bad);
   return bad ? 1 : 0;
 }
