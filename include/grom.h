@@ -484,8 +484,9 @@ grom_status grom_als_fit(grom_als* als, int32_t rank, int32_t method, int32_t it
                          double ridge, double* fa, double* fb, double* fc, double* residual);
 /* Time spent since the previous call: summed device time of the MTTKRP
  * launches (CUDA events around each tensor-core launch), their number, and
- * the wall time of the SPD solves, each from its first launch to its end on
- * the device (ms).  Resets the counters. */
+ * the device time of the SPD solves (ms): every factorisation from its first
+ * launch to its end, also where it runs beside an MTTKRP, and the triangular
+ * solves.  Resets the counters. */
 grom_status grom_als_stats(grom_als* als, double* mttkrp_ms, int64_t* mttkrp_calls, double* solve_ms);
 grom_status grom_als_destroy(grom_als* als);
 

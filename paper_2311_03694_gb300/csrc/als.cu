@@ -52,11 +52,11 @@ struct grom_als {
   void* k2s = nullptr;
   size_t k2s_bytes = 0;
   // timing since the last grom_als_stats: device times (CUDA events) of the
-  // tensor-core launches and of the SPD solves (the part of a factorisation
-  // that outlasts its MTTKRP, and the triangular solves)
+  // tensor-core launches and of the SPD solves (each factorisation from its
+  // first launch, whatever runs beside it, and the triangular solves)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   cudaStream_t side = nullptr;                    // the factorisations' stream
-  cudaEvent_t fork = nullptr, join = nullptr, sv0 = nullptr, sv1 = nullptr;
+  cudaEvent_t fork = nullptr, sf0 = nullptr, join = nullptr, sv0 = nullptr, sv1 = nullptr;
   double mttkrp_ms = 0.0, solve_ms = 0.0;
   int64_t mttkrp_calls = 0;
 };
@@ -658,11 +658,12 @@ grom_status ls_update(grom_als* s, int m, int fp, int fq, int64_t r, double ridg
   grom_status st;
   GROM_CUDA_TRY(cudaEventRecord(s->fork, s->stream));
   GROM_CUDA_TRY(cudaStreamWaitEvent(s->side, s->fork, 0));
+  GROM_CUDA_TRY(cudaEventRecord(s->sf0, s->side));
   if ((st = factorise(s, Ga, Gb, r, ridge, s->side))) return st;
   GROM_CUDA_TRY(cudaEventRecord(s->join, s->side));
   if (!have_m && (st = mttkrp(s, m, fp, fq, r))) return st;
-  GROM_CUDA_TRY(cudaEventRecord(s->sv0, s->stream));
   GROM_CUDA_TRY(cudaStreamWaitEvent(s->stream, s->join, 0));
+  GROM_CUDA_TRY(cudaEventRecord(s->sv0, s->stream));
   bool ok = false, ran = !have_m;
   double mu = 0.0;
   for (int attempt = 0; attempt < 4 && !ok; ++attempt) {
@@ -677,6 +678,8 @@ grom_status ls_update(grom_als* s, int m, int fp, int fq, int64_t r, double ridg
   }
   if (!ok) return fail(GROM_ERR_INVALID_ARG, "grom_als_fit: a Gram matrix is not positive definite");
   float ms = 0.f;
+  GROM_CUDA_TRY(cudaEventElapsedTime(&ms, s->sf0, s->join));
+  s->solve_ms += ms;
   GROM_CUDA_TRY(cudaEventElapsedTime(&ms, s->sv0, s->sv1));
   s->solve_ms += ms;
   if (dst != s->anew)
@@ -746,7 +749,7 @@ grom_status grom_als_create(int32_t n, const double* tensor, void* stream, grom_
   if (cudaEventCreate(&s->ev0) != cudaSuccess || cudaEventCreate(&s->ev1) != cudaSuccess ||
       cudaEventCreate(&s->sv0) != cudaSuccess || cudaEventCreate(&s->sv1) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreate(&s->sf0) != cudaSuccess || cudaEventCreate(&s->join) != cudaSuccess ||
       cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) != cudaSuccess)
     return bail(cuda_fail(cudaGetLastError(), "grom_als_create: events"));
   // stream the FP64 tensor through a staging buffer by test index
@@ -866,7 +869,7 @@ grom_status grom_als_destroy(grom_als* s) {
   if (!s) return GROM_OK;
   if (s->side) cudaStreamSynchronize(s->side);
   if (s->stream) cudaStreamSynchronize(s->stream);
-  for (cudaEvent_t e : {s->ev0, s->ev1, s->sv0, s->sv1, s->fork, s->join})
+  for (cudaEvent_t e : {s->ev0, s->ev1, s->sf0, s->sv0, s->sv1, s->fork, s->join})
     if (e) cudaEventDestroy(e);
   if (s->side) cudaStreamDestroy(s->side);
   for (auto p : s->x)
