@@ -167,6 +167,7 @@ struct K2PPlan {
   int wrows;       // rows of the mirrored-entry window (m + 127)
   int wpitch;      // its pitch in floats (btile + 1)
   int grid;        // persistent CTAs (pairs: even, at most the pairs that fit at once)
+  int sm_count;    // of the device the plan is for
   int64_t bp;      // padded batch
   size_t smem;
 };

@@ -577,9 +577,16 @@ __global__ void k2p_prep_kernel(const K2PDev p, float* uf, __nv_bfloat16* uh, __
 // index's 32 trajectories (128-byte lines), the totals turn through shared
 // memory and the rows of c are written 128 bytes at a time, with 32-bit index
 // arithmetic and independent loads (n = 1024, 1024 trajectories: 79.7 us
-// against 96.4).  Reading the 123 MB of partial sums once is its floor (18 us).
-constexpr int K2PF_K = 16, K2PF_B = 32, K2PF_WARPS = 8;
-__global__ void __launch_bounds__(32 * K2PF_WARPS)
+// against 96.4 with a thread per output).  Reading the 123 MB of partial sums
+// once is its floor (18 us).  With fewer than about two blocks an SM the chain
+// of one test index after the other in a warp is what takes the time, and a
+// block has a warp for each of its 16.  us with 8 and with 16 warps: n = 50, 94
+// trajectories 15.5, 7.1 (a thread per output 9.0); n = 900, 12 18.8, 11.2
+// (16.0); n = 512, 256 11.9, 8.8; n = 256, 1024 (512 blocks) 9.4, 10.2; n =
+// 1024, 1024 79.7, 100.6.
+constexpr int K2PF_K = 16, K2PF_B = 32;
+template <int WARPS>
+__global__ void __launch_bounds__(32 * WARPS)
     k2p_finish_kernel(const K2PDev p, double* c, int64_t c_stride, double* hist, const int64_t* taken,
                       int64_t hist_stride, const int32_t* active, int batch) {
   __shared__ double sh[K2PF_B][K2PF_K + 1];
@@ -588,7 +595,7 @@ __global__ void __launch_bounds__(32 * K2PF_WARPS)
   const int k0 = blockIdx.x * K2PF_K, b0 = blockIdx.y * K2PF_B, b = b0 + lane;
   const int ct = b / p.btile, bl = b - ct * p.btile;
   const int64_t tile = (int64_t)wrows * p.btile;
-  for (int kq = warp; kq < K2PF_K; kq += K2PF_WARPS) {
+  for (int kq = warp; kq < K2PF_K; kq += WARPS) {
     const int k = k0 + kq;
     if (k >= n || b >= batch) continue;
     float sd = 0.f, sm = 0.f;
@@ -627,7 +634,7 @@ __global__ void __launch_bounds__(32 * K2PF_WARPS)
     sh[lane][kq] = (double)sd - (double)sm;
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < K2PF_K * K2PF_B; t += 32 * K2PF_WARPS) {
+  for (int t = threadIdx.x; t < K2PF_K * K2PF_B; t += 32 * WARPS) {
     const int64_t k = k0 + t % K2PF_K, bt = b0 + t / K2PF_K;
     if (k >= n || bt >= batch || (active && !active[bt])) continue;
     double* dst = taken ? hist + bt * hist_stride + (3 + taken[bt] % 3) * p.n : c + bt * c_stride;
@@ -698,6 +705,7 @@ K2PPlan k2p_plan(int64_t n, int64_t lp, int batch, int sm_count, int m_force, in
   p.n = n;
   p.np = padded_n(n);
   p.lp = lp;
+  p.sm_count = sm_count;
   const int btile = k2p_btile(batch);
   p.btile = btile;
   p.col_tiles = (batch + btile - 1) / btile;
@@ -843,8 +851,10 @@ cudaError_t k2p_launch(const K2PPlan& p, const CUtensorMap* tmap, const K2Args& 
   if (e != cudaSuccess) return e;
   if (a.ev1) prof_record(a.ev1, s);
   const dim3 fin((unsigned)((p.n + K2PF_K - 1) / K2PF_K), (unsigned)((a.batch + K2PF_B - 1) / K2PF_B));
-  k2p_finish_kernel<<<fin, 32 * K2PF_WARPS, 0, s>>>(d, a.c, a.c_stride, a.hist, a.taken, a.hist_stride, a.active,
-                                                    a.batch);
+  if ((int64_t)fin.x * fin.y < 2 * p.sm_count)
+    k2p_finish_kernel<16><<<fin, 512, 0, s>>>(d, a.c, a.c_stride, a.hist, a.taken, a.hist_stride, a.active, a.batch);
+  else
+    k2p_finish_kernel<8><<<fin, 256, 0, s>>>(d, a.c, a.c_stride, a.hist, a.taken, a.hist_stride, a.active, a.batch);
   return cudaGetLastError();
 }
 
