@@ -338,6 +338,11 @@ __global__ void __launch_bounds__(K1_THREADS, 1)
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
           if (b >= nb) break;
+          const int64_t l = l0s[b] + step;
+          const int k = (int)(l + 1 < st.order ? l + 1 : st.order);
+          double* h = st.hist + b * st.hist_stride;
+          StepElem x{};
+          if (lane == 0) x = step_load(st, h, n, l, k, i);
           double v = 0.0;
           for (int q = lane; q < nrp; q += 32) {  // row sums of the CTAs covering i
             const int64_t go = g_lo + q / (K1_CONSUMERS / 32);
@@ -353,13 +358,10 @@ __global__ void __launch_bounds__(K1_THREADS, 1)
 #pragma unroll
           for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
           if (lane == 0) {
-            const int64_t l = l0s[b] + step;
-            const int k = (int)(l + 1 < st.order ? l + 1 : st.order);
-            double* h = st.hist + b * st.hist_stride;
             h[(3 + l % 3) * n + i] = v;
             double ep, ip;
             int bb;
-            step_elem(st, h, n, l, k, i, v, ep, ip, bb);
+            step_elem(st, h, n, l, k, i, x, v, ep, ip, bb);
             ew[b] += ep;
             iw[b] += ip;
             if (bb) {

@@ -508,7 +508,9 @@ __global__ void __launch_bounds__(K1T_THREADS, 1) k1t_kernel(const K1TArgs a, co
               h[(3 + l % 3) * n + i] = v;
               double ep, ip;
               int bb;
-              step_elem(st, h, n, l, k, i, v, ep, ip, bb);
+              // (loaded before the windows, these operands cost the F32X2
+              // stream 2 %: 435 us a step of n = 1024 against 444)
+              step_elem(st, h, n, l, k, i, step_load(st, h, n, l, k, i), v, ep, ip, bb);
               ew[b] += ep;
               iw[b] += ip;
               if (bb) {

@@ -228,6 +228,9 @@ __global__ void __launch_bounds__(STEP_PK_THREADS) k_step_diag_packed(const Step
   for (int g = threadIdx.x; g < G; g += blockDim.x) fi_tab[g] = (int)(((int64_t)g * T / G) / pl.cpi);
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+  const int64_t l = a.taken[b];
+  const int k = (int)(l + 1 < a.order ? l + 1 : a.order);
+  double* h = a.hist + b * a.hist_stride;
   double s = 0.0;
   if (i < n) {
     const int g0 = warp * G / 32, g1 = (warp + 1) * G / 32;
@@ -257,7 +260,9 @@ __global__ void __launch_bounds__(STEP_PK_THREADS) k_step_diag_packed(const Step
   }
   sh[warp][lane] = s;
   double rs = 0.0;
+  StepElem x{};
   if (warp == 0 && i < n) {
+    x = step_load(a, h, n, l, k, i);
     const int64_t g_lo = ((i * pl.cpi + 1) * G - 1) / T, g_hi = (((i + 1) * pl.cpi) * G - 1) / T;
     for (int64_t g = g_lo; g <= g_hi; ++g) {
       const double* src = k1a.part + ((g * pl.maxseg + (i - fi_tab[g])) * (K1_CONSUMERS / 32)) * nbk + bl;
@@ -270,9 +275,6 @@ __global__ void __launch_bounds__(STEP_PK_THREADS) k_step_diag_packed(const Step
   }
   __syncthreads();
   if (warp != 0) return;
-  const int64_t l = a.taken[b];
-  const int k = (int)(l + 1 < a.order ? l + 1 : a.order);
-  double* h = a.hist + b * a.hist_stride;
   double e_part = 0.0, i_part = 0.0;
   int bad = 0;
   if (i < n) {
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(STEP_PK_THREADS) k_step_diag_packed(const Step
     for (int w = 0; w < 32; ++w) t += sh[w][lane];
     const double nl = rs - t;
     h[(3 + l % 3) * n + i] = nl;
-    step_elem(a, h, n, l, k, i, nl, e_part, i_part, bad);
+    step_elem(a, h, n, l, k, i, x, nl, e_part, i_part, bad);
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {

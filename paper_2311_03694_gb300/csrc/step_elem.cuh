@@ -56,44 +56,59 @@ __device__ __forceinline__ int step_is_bad(double un) {  // inf or NaN, from the
 // those terms at compile time: a runtime test still issues its predicated
 // FP64 instructions, which measured ~26 FP64 instructions per element on the
 // batched step.
+// The operands other than the newest advection term are loaded by step_load,
+// which the kernels call before they sum that term, so that both loads' latencies
+// pass together; a lower order leaves some unused.
+struct StepElem {
+  double u[3], g[3], hd, mb, ld, f;
+};
 template <bool PLAIN = false>
-__device__ __forceinline__ double step_elem(const StepArgs& a, double* h, int64_t n, int64_t l, int k, int64_t i,
-                                            double nl, double& e_part, double& i_part, int& bad, bool sums = true) {
-  const bool lin = !PLAIN && a.lin_diag != nullptr, frc = !PLAIN && a.forcing != nullptr,
-             mass = !PLAIN && a.mass_diag != nullptr;
-  if (PLAIN) sums = false;
-  const double ld = lin ? a.lin_diag[i] : 0.0;
-  const double f = frc ? a.forcing[i] : 0.0;
+__device__ __forceinline__ StepElem step_load(const StepArgs& a, const double* h, int64_t n, int64_t l, int k,
+                                              int64_t i) {
+  StepElem x;
   const int m0 = (int)(l % 3);
-  double u[3] = {0.0, 0.0, 0.0}, g[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    if (PLAIN || q < k) {  // plain: all six loads in flight at once, a lower order leaves some unused
-      const int m = m0 - q < 0 ? m0 - q + 3 : m0 - q;
-      u[q] = h[m * n + i];
-      g[q] = q == 0 ? nl : h[(3 + m) * n + i];
-      if (lin) g[q] = fma(ld, u[q], g[q]);
-      if (frc) g[q] += f;
-    }
+    const int m = m0 - q < 0 ? m0 - q + 3 : m0 - q;
+    x.u[q] = h[m * n + i];
+    x.g[q] = q == 0 ? 0.0 : h[(3 + m) * n + i];
   }
-  double un, mb = 1.0;
+  x.hd = a.hdiag[k - 1][i];
+  x.mb = !PLAIN && a.mass_diag ? a.mass_diag[i] : 1.0;
+  x.ld = !PLAIN && a.lin_diag ? a.lin_diag[i] : 0.0;
+  x.f = !PLAIN && a.forcing ? a.forcing[i] : 0.0;
+  return x;
+}
+template <bool PLAIN = false>
+__device__ __forceinline__ double step_elem(const StepArgs& a, double* h, int64_t n, int64_t l, int k, int64_t i,
+                                            const StepElem& x, double nl, double& e_part, double& i_part, int& bad,
+                                            bool sums = true) {
+  const bool mass = !PLAIN && a.mass_diag != nullptr;
+  const bool lin = !PLAIN && a.lin_diag != nullptr;
+  const bool frc = !PLAIN && a.forcing != nullptr;
+  double g[3] = {nl, x.g[1], x.g[2]};
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (lin) g[q] = fma(x.ld, x.u[q], g[q]);
+    if (frc) g[q] += x.f;
+  }
+  double un;
   if (mass) {
-    mb = a.mass_diag[i];
     double bdf = 0.0;
 #pragma unroll
     for (int q = 0; q < 3; ++q)
-      if (q < k) bdf = fma(a.bdt[k - 1][q], u[q], bdf);
-    un = fma(-mb, bdf, -step_ext(k, g)) * a.hdiag[k - 1][i];
+      if (q < k) bdf = fma(a.bdt[k - 1][q], x.u[q], bdf);
+    un = fma(-x.mb, bdf, -step_ext(k, g)) * x.hd;
   } else {
-    un = step_plain_elem(a.bdt[k - 1], k, u, g, a.hdiag[k - 1][i]);
+    un = step_plain_elem(a.bdt[k - 1], k, x.u, g, x.hd);
   }
   e_part = 0.0;
   i_part = 0.0;
   if (sums) {
     // explicit roundings: the products must not contract into the caller's
     // sums (FMA), whose form would then depend on the kernel inlining them
-    e_part = mass ? __dmul_rn(__dmul_rn(mb, un), un) : __dmul_rn(un, un);
-    i_part = __dmul_rn(u[0], nl);
+    e_part = mass ? __dmul_rn(__dmul_rn(x.mb, un), un) : __dmul_rn(un, un);
+    i_part = __dmul_rn(x.u[0], nl);
   }
   bad = step_is_bad(un);
   h[((l + 1) % 3) * n + i] = un;

@@ -73,6 +73,7 @@ __device__ __forceinline__ void step_mc_block(const StepArgs& a, int step_index,
   for (int e = 0; e < a.ept; ++e) {
     const int64_t i = ((int64_t)blk * a.ept + e) * STEP_MC_THREADS + tid;
     if (i >= n) break;
+    const StepElem x = step_load<PLAIN>(a, h, n, l, k, i);
     double nl;
     if (fuse == 3) {
       // expansion splits in split order, double-single (as the K3D finish)
@@ -121,7 +122,7 @@ __device__ __forceinline__ void step_mc_block(const StepArgs& a, int step_index,
     }
     double ep, ip;
     int eb;
-    const double un = step_elem<PLAIN>(a, h, n, l, k, i, nl, ep, ip, eb, sums);
+    const double un = step_elem<PLAIN>(a, h, n, l, k, i, x, nl, ep, ip, eb, sums);
     if (fuse == 3) {
       float hi, lo;
       ds_split(un, hi, lo);
