@@ -1310,13 +1310,13 @@ grom_status grom_step(grom_traj* t, int32_t nsteps, double* energy, double* inva
   // cannot be placed)
   if (r->diagonal && is_cp(r) && !t->active && !r->prof && nsteps >= 4 && !use_k3t(r, t->batch, false)) {
     const uint8_t *fa = r->op, *fb = r->op + r->panel_bytes, *fc = r->op + 2 * r->panel_bytes;
-    const bool few = t->batch <= k3p_max_batch(r->storage);
     const StepArgs a = step_args(t, energy, invariant);
     cudaError_t e = cudaErrorNotSupported;
-    if (few && k3x_fits(r->n, r->k3.rb, r->form, r->storage, t->batch, r->sm_count))
+    if (k3x_fits(r->n, r->k3.rb, r->form, r->storage, t->batch, r->sm_count))
       e = k3x_launch(fa, fb, fc, r->form, r->n, r->k3.rb, r->storage, t->batch, nsteps, a, r->k3x_scratch, r->sm_count,
                      r->stream);
-    if (not_placed(e) && few && k3p_fits(r->n, r->k3.rb, r->storage, t->batch, r->sm_count))
+    if (not_placed(e) && t->batch <= k3p_max_batch(r->storage) &&
+        k3p_fits(r->n, r->k3.rb, r->storage, t->batch, r->sm_count))
       e = k3p_launch(fa, fb, fc, r->form, r->n, r->k3.rb, r->storage, t->batch, nsteps, a, r->k3p_scratch, r->sm_count,
                      r->stream);
     if (e == cudaSuccess) return GROM_OK;

@@ -177,7 +177,7 @@ cudaError_t k1tp_launch(const K1TPlan& p, K1TArgs a, const StepArgs& st, int bat
 // reads run along the tensor's last index, the writes along p.
 constexpr int T_P = 16, T_Q = 16, T_M = 8;
 __global__ void __launch_bounds__(256) k1t_convert_kernel(const double* __restrict__ src, const int n,
-                                                          const int64_t* __restrict__ off, const int epv, const int i0,
+                                                          const int64_t* __restrict__ off, const int i0,
                                                           const int cnt, const int x2, uint8_t* __restrict__ dst) {
   __shared__ double A[T_P][T_Q * T_M + 1], B[T_P][T_M * T_Q + 1];
   const int m0 = blockIdx.x * T_M, q0 = blockIdx.y * T_Q, pl0 = blockIdx.z * T_P;
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(256) k1t_convert_kernel(const double* __restri
 
 cudaError_t k1t_convert(const K1TPlan& p, const double* src, int64_t i0, int64_t cnt, uint8_t* dst, cudaStream_t s) {
   const dim3 grid((unsigned)((p.n + T_M - 1) / T_M), (unsigned)((p.n + T_Q - 1) / T_Q), (unsigned)((cnt + T_P - 1) / T_P));
-  k1t_convert_kernel<<<grid, 256, 0, s>>>(src, p.n, p.d_off, p.epv, (int)i0, (int)cnt, p.storage == GROM_F32X2, dst);
+  k1t_convert_kernel<<<grid, 256, 0, s>>>(src, p.n, p.d_off, (int)i0, (int)cnt, p.storage == GROM_F32X2, dst);
   return cudaGetLastError();
 }
 

@@ -12,14 +12,14 @@
 // largest.  Each stored value is one FP64 sum of two entries, rounded once
 // into the storage.)  u . c = 0 holds term by term, as for the entries
 // themselves.  Against one entry of each pair (n^3 / 2) the bytes and the
-// multiply-adds are two thirds: a step of n = 1024 F32X2, bound by HBM (2.87
+// multiply-adds are two thirds: a step of n = 1024 F32X2, bound by HBM (2.89
 // GB at 6.6 TB/s), takes 433 us instead of 650; an evaluation of n = 769 F64,
 // three trajectories, bound by the FP64 pipe (0.7 ms of it at two
 // multiply-adds a clock and SM), 975 us instead of 1759.
 //
-// Group m holds m + 1 rows q of the m values p (p contiguous, zero-padded to
-// a 16-byte vector; F32X2: the hi values, then the lo ones), and starts on a
-// 128-byte boundary.  A CTA streams a contiguous range of rows through a ring
+// Group m holds m + 1 rows q of the m values p (p contiguous; F32X2: the hi
+// values, then the lo ones), each zero-padded to 128 bytes, so that every row
+// starts on such a boundary.  A CTA streams a contiguous range of rows through a ring
 // of bulk copies; a consumer thread owns positions p and accumulates D_p over
 // the rows, so nothing is reduced per row.  At the end of a group it adds
 // D_p u_m to its own c_p, kept for the whole range, and the warp sums D_p u_p;
@@ -404,10 +404,6 @@ __global__ void __launch_bounds__(K1T_THREADS, 1) k1t_kernel(const K1TArgs a, co
             case 2: if constexpr (QM >= 2) take(std::integral_constant<int, 2>()); break;
             case 3: if constexpr (QM >= 4) take(std::integral_constant<int, 3>()); break;
             case 4: if constexpr (QM >= 4) take(std::integral_constant<int, 4>()); break;
-            case 5: if constexpr (QM >= 8) take(std::integral_constant<int, 5>()); break;
-            case 6: if constexpr (QM >= 8) take(std::integral_constant<int, 6>()); break;
-            case 7: if constexpr (QM >= 8) take(std::integral_constant<int, 7>()); break;
-            case 8: if constexpr (QM >= 8) take(std::integral_constant<int, 8>()); break;
           }
         }
         if (stop) break;

@@ -62,7 +62,7 @@ struct K1TArgs {
   const int64_t* off;
   const int4* ranges;
   int n, np, stages, maxseg;
-  double* part;  // grid x maxseg x 8 warps x NB row sums
+  double* part;  // grid x maxseg x K1T_WARPS x NB row sums
   double* win;   // grid x NB x np windows of c
   int nb, b0;    // trajectories of this pass, the first one
   int nsteps;    // 0: one evaluation

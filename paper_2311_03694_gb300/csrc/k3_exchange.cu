@@ -1,6 +1,6 @@
-// Persistent CPD-ROM stepper for one to four trajectories whose factors fit
-// the shared memory of the chip twice over: every step of a grom_step call in
-// one cooperative launch, without grid barriers.
+// Persistent CPD-ROM stepper for one to four trajectories (F64: one or two)
+// whose factors fit the shared memory of the chip twice over: every step of a
+// grom_step call in one cooperative launch, without grid barriers.
 //
 // CTA g keeps its rank columns of the projected factors and its rows of the
 // expansion factors in shared memory.  A step:
@@ -524,8 +524,8 @@ __global__ void __launch_bounds__(KX_THREADS, 1) k3x_kernel(const KXArgs p) {
 
 // ------------------------------------------------------------- evaluations
 // One evaluation of FP64 factors with the same exchange: the CTAs' columns
-// straight from memory (a thread takes whole pieces of a factor's rows; the
-// rows of the expansion are copied to shared memory meanwhile), h published,
+// straight from memory (a thread takes the CTA's entries of every 256th row of
+// a factor; the rows of the expansion are copied to shared memory meanwhile), h published,
 // then the CTAs' rows.  The two kernels of k3_cp.cu cost a second launch, the
 // row slices' partial sums and their gathering; here one exchange is left, and
 // the rest is latency.  us an evaluation, here against two kernels: n = 500,
@@ -700,8 +700,10 @@ static KXShape kx_shape(int64_t n, int64_t rp, int form, int storage, int batch,
   return s;
 }
 
+// Trajectories of a launch; FP64 ROMs step three and four through the per-step kernels.
+static constexpr int kx_max_batch(int storage) { return storage == GROM_F64 ? 2 : 4; }
 bool k3x_fits(int64_t n, int64_t rp, int form, int storage, int batch, int sm_count) {
-  if (batch > 4 || n > (1 << 14) || rp > (1 << 14)) return false;
+  if (batch > kx_max_batch(storage) || n > (1 << 14) || rp > (1 << 14)) return false;
   return kx_shape(n, rp, form, storage, batch, sm_count).smem <= 220 * 1024;
 }
 
@@ -712,7 +714,7 @@ size_t k3x_scratch_bytes(int64_t n, int64_t rp, int sm_count) {
 
 template <int ST>
 static cudaError_t kx_run(const KXArgs& p, const KXShape& s, cudaStream_t strm) {
-  auto kern = s.nb == 1 ? k3x_kernel<ST, 1> : s.nb == 2 ? k3x_kernel<ST, 2> : k3x_kernel<ST, 4>;
+  auto kern = s.nb == 1 ? k3x_kernel<ST, 1> : s.nb == 2 ? k3x_kernel<ST, 2> : k3x_kernel<ST, kx_max_batch(ST)>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem);
   if (e != cudaSuccess) return e;
   KXArgs a = p;
