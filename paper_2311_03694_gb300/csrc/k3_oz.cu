@@ -338,25 +338,47 @@ __device__ __forceinline__ void oz_sum(const float* __restrict__ D, int64_t M, i
   }
 }
 
-// The pairs of one output from k3_tri.cu, [split][hi, lo][bq][M], in split order.
+// The pairs of one output from k3_tri.cu, [split][hi, lo][bq][M], in split
+// order, in three floats: as double-single sums each split added two roundings of
+// the pair's last bit (n = 1024, r = 512, 64 trajectories, against long double,
+// median over the states: 5.6e-15 an evaluation, 2.0e-15 this way).  G splits'
+// loads in flight: eight for tiles of more than four splits in grids that fit the
+// device at once (oz_wide), which wait for the loads; else four, whose registers
+// leave room for twice the warps (n = r = 1024, 1024 trajectories, a step: 466 us
+// with eight, 440 with four; r = 512, 64 trajectories 39.1 and 42.5).  FILL: zeros
+// for the splits that are not there, so that the sums' chains overlap without
+// branches between them (k3o_exp_step at 64 trajectories 8.2 -> 7.9 us; the two
+// combine kernels lose 0.5 us with it, their loads then come one after the other).
+template <int G, bool FILL>
 __device__ __forceinline__ void oz_sum_tri(const float* __restrict__ D, int splits, int64_t M, int64_t bq, int b,
                                            int64_t m, float& S, float& s) {
   const int64_t plane = bq * M;
   const float* p = D + (int64_t)b * M + m;
-  S = 0.f;
-  s = 0.f;
-  for (int q0 = 0; q0 < splits; q0 += 8) {  // eight splits' loads in flight
-    float v[8][2];
+  float s1 = 0.f, s2 = 0.f, s3 = 0.f;
+  for (int q0 = 0; q0 < splits; q0 += G) {
+    float v[G][2];
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
+    for (int k = 0; k < G; ++k) {
+      if constexpr (FILL) v[k][0] = v[k][1] = 0.f;
       if (q0 + k < splits) {
         v[k][0] = __ldcg(p + (int64_t)(q0 + k) * 2 * plane);
         v[k][1] = __ldcg(p + (int64_t)(q0 + k) * 2 * plane + plane);
       }
+    }
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (q0 + k < splits) ds_add(S, s, v[k][0], v[k][1]);
+    for (int k0 = 0; k0 < G; k0 += 4) {
+      if (FILL && q0 + k0 >= splits) break;
+#pragma unroll
+      for (int k = k0; k < k0 + 4; ++k)
+        if (FILL || q0 + k < splits) {
+          ts_add(v[k][0], s1, s2, s3);
+          ts_add_low(v[k][1], s2, s3);
+        }
+    }
   }
+  S = __fadd_rn(s1, s2);
+  s = __fadd_rn(__fsub_rn(s2, __fsub_rn(S, s1)), s3);
+  ds_renorm(S, s);
 }
 
 // (S, s) times 2^e, exactly (e in the FP32 exponent range).
@@ -371,7 +393,8 @@ __device__ __forceinline__ void oz_scale_ds(float& S, float& s, int e) {
 // (and H2 = P o S) as double-single pairs and the bits of the trajectory's
 // largest |H hi|.  (Three threads per output keep three times the loads in
 // flight of one thread per (b, j).)
-template <int S, int BITS>
+// G: 8 or 4 as in oz_sum_tri.
+template <int S, int BITS, int G>
 __global__ void __launch_bounds__(192) k3o_combine_proj(const ODims d, const float* __restrict__ D1,
                                                         const int* __restrict__ sproj, const int* __restrict__ tau,
                                                         float* Hh, float* Hl, unsigned int* hmax, const int splits) {
@@ -386,7 +409,7 @@ __global__ void __launch_bounds__(192) k3o_combine_proj(const ODims d, const flo
     const int64_t m = (int64_t)f * d.r + j;
     float hi, lo;
     if constexpr (S == OZ_S7)
-      oz_sum_tri(D1, splits, d.mp, d.bq, b, m, hi, lo);
+      oz_sum_tri<G, false>(D1, splits, d.mp, d.bq, b, m, hi, lo);
     else
       oz_sum<S, BITS>(D1, M, d.mp, d.bq, b, m, hi, lo);
     oz_scale_ds(hi, lo, sproj[m] + tau[b]);
@@ -440,6 +463,7 @@ __global__ void __launch_bounds__(256) k3o_slice_h(const ODims d, const K3Args a
 }
 
 // One thread per (b, i), i fastest: c_bi into the output or the ring.
+template <int G>
 __global__ void __launch_bounds__(256) k3o_combine_exp(const ODims d, const K3Args a, const float* __restrict__ D2,
                                                        const int* __restrict__ sexp, const int* __restrict__ tau2,
                                                        const int splits) {
@@ -452,7 +476,7 @@ __global__ void __launch_bounds__(256) k3o_combine_exp(const ODims d, const K3Ar
     if (a.active && !a.active[b]) continue;
     float S, s;
     if (splits)
-      oz_sum_tri(D2, splits, d.me, d.bq, b, i, S, s);
+      oz_sum_tri<G, false>(D2, splits, d.me, d.bq, b, i, S, s);
     else
       oz_sum<OZ_S, OZ_BITS>(D2, M, d.me, d.bq, b, i, S, s);
     oz_scale_ds(S, s, sexp[i] + tau2[b]);
@@ -467,7 +491,7 @@ __global__ void __launch_bounds__(256) k3o_combine_exp(const ODims d, const K3Ar
 // writes it into the history ring; each thread then reads back only what it
 // wrote itself.  One launch and one pass over c fewer than the combine
 // followed by the step kernel, with the same bits.
-template <bool PLAIN>
+template <bool PLAIN, int G>
 __global__ void __launch_bounds__(STEP_MC_THREADS)
     k3o_exp_step(const ODims d, const float* __restrict__ D2, const int* __restrict__ sexp,
                  const int* __restrict__ tau2, const int splits, const StepArgs st, const int step_index) {
@@ -485,7 +509,7 @@ __global__ void __launch_bounds__(STEP_MC_THREADS)
       if (i >= d.n) break;
       float S, s;
       if (splits)
-        oz_sum_tri(D2, splits, d.me, d.bq, b, i, S, s);
+        oz_sum_tri<G, true>(D2, splits, d.me, d.bq, b, i, S, s);
       else
         oz_sum<OZ_S, OZ_BITS>(D2, M, d.me, d.bq, b, i, S, s);
       oz_scale_ds(S, s, sexp[i] + tau2[b]);
@@ -535,6 +559,8 @@ static unsigned oz_flat_blocks(int64_t count, int sm_count) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(b, 8 * (int64_t)sm_count));
 }
 
+static bool oz_wide(int splits, int64_t blocks, int sm_count) { return splits > 4 && blocks <= 4 * sm_count; }
+
 // Everything up to the expansion GEMM (digit slices of the states, the
 // projections and their combine, the slices of [H1 H2], the expansion's
 // slice products in d2); returns d2 and the expansion scales.
@@ -569,7 +595,9 @@ static cudaError_t k3o_front(const ODims& d, const K3Args& a, const void* factor
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = k3o_tri_launch(fb + F.aproj, d.mp, bst, d.bq, d.nk, d1, err, sm_count, s);
     if (e == cudaSuccess)
-      e = launch_dependent(k3o_combine_proj<OZ_S7, OZ_BITS7>, gc, 192, 0, s, d, d1, spj, tau, hh, hl, hmax, s1);
+      e = launch_dependent(oz_wide(s1, (int64_t)gc.x * gc.y, sm_count) ? k3o_combine_proj<OZ_S7, OZ_BITS7, 8>
+                                                                   : k3o_combine_proj<OZ_S7, OZ_BITS7, 4>,
+                           gc, 192, 0, s, d, d1, spj, tau, hh, hl, hmax, s1);
     if (e == cudaSuccess)
       e = launch_dependent(k3o_slice_h<OZ_S7, OZ_BITS7>, gh, 256, 0, s, d, a, hh, hl, hmax, bh, tau2);
     return e == cudaSuccess ? k3o_tri_launch(fb + F.aexp, d.me, bh, d.bq, d.rk, d2, err, sm_count, s) : e;
@@ -578,7 +606,7 @@ static cudaError_t k3o_front(const ODims& d, const K3Args& a, const void* factor
   cudaError_t e = k3o_gemm_launch(fb + F.aproj, (int64_t)d.sp * d.mp, d.mp, bst, d.ncp, d.bq, d.nk, d.sp, d1, err,
                                   sm_count, s);
   if (e != cudaSuccess) return e;
-  k3o_combine_proj<OZ_S, OZ_BITS><<<gc, 192, 0, s>>>(d, d1, spj, tau, hh, hl, hmax, 0);
+  k3o_combine_proj<OZ_S, OZ_BITS, 4><<<gc, 192, 0, s>>>(d, d1, spj, tau, hh, hl, hmax, 0);
   k3o_slice_h<OZ_S, OZ_BITS><<<gh, 256, 0, s>>>(d, a, hh, hl, hmax, bh, tau2);
   return k3o_gemm_launch(fb + F.aexp, OZ_S * d.me, d.me, bh, d.nc, d.bq, d.rk, OZ_S, d2, err, sm_count, s);
 }
@@ -592,8 +620,10 @@ cudaError_t k3o_launch(int64_t n, int64_t rp, int64_t r, const K3Args& a, const 
   cudaError_t e = k3o_front(d, a, factors, scratch, err, sm_count, s, &d2, &sexp, &tau2, &s2);
   if (e != cudaSuccess) return e;
   const unsigned blocks = oz_flat_blocks((int64_t)batch * d.n, sm_count);
-  if (s2) return launch_dependent(k3o_combine_exp, dim3(blocks), 256, 0, s, d, a, d2, sexp, tau2, s2);
-  k3o_combine_exp<<<blocks, 256, 0, s>>>(d, a, d2, sexp, tau2, s2);
+  if (s2)
+    return launch_dependent(oz_wide(s2, blocks, sm_count) ? k3o_combine_exp<8> : k3o_combine_exp<4>, dim3(blocks), 256, 0, s,
+                            d, a, d2, sexp, tau2, s2);
+  k3o_combine_exp<4><<<blocks, 256, 0, s>>>(d, a, d2, sexp, tau2, s2);
   return cudaGetLastError();
 }
 
@@ -611,13 +641,16 @@ cudaError_t k3o_launch_step(int64_t n, int64_t rp, int64_t r, const K3Args& a, c
   st1.ept = 1;
   st1.nblk = step_mc_blocks(n);
   const dim3 grid((unsigned)st1.nblk, (unsigned)batch);
-  if (s2)
-    return step_plain(st1) ? launch_dependent(k3o_exp_step<true>, grid, STEP_MC_THREADS, 0, s, d, d2, sexp, tau2, s2, st1, step_index)
-                           : launch_dependent(k3o_exp_step<false>, grid, STEP_MC_THREADS, 0, s, d, d2, sexp, tau2, s2, st1, step_index);
+  if (s2) {
+    const bool wide = oz_wide(s2, (int64_t)grid.x * grid.y, sm_count);
+    return launch_dependent(step_plain(st1) ? (wide ? k3o_exp_step<true, 8> : k3o_exp_step<true, 4>)
+                                            : (wide ? k3o_exp_step<false, 8> : k3o_exp_step<false, 4>),
+                            grid, STEP_MC_THREADS, 0, s, d, d2, sexp, tau2, s2, st1, step_index);
+  }
   if (step_plain(st1))
-    k3o_exp_step<true><<<grid, STEP_MC_THREADS, 0, s>>>(d, d2, sexp, tau2, s2, st1, step_index);
+    k3o_exp_step<true, 4><<<grid, STEP_MC_THREADS, 0, s>>>(d, d2, sexp, tau2, s2, st1, step_index);
   else
-    k3o_exp_step<false><<<grid, STEP_MC_THREADS, 0, s>>>(d, d2, sexp, tau2, s2, st1, step_index);
+    k3o_exp_step<false, 4><<<grid, STEP_MC_THREADS, 0, s>>>(d, d2, sexp, tau2, s2, st1, step_index);
   return cudaGetLastError();
 }
 
