@@ -130,13 +130,6 @@ __device__ __forceinline__ void ts_add(float v, float& s1, float& s2, float& s3)
   s3 = __fadd_rn(s3, e2);
 }
 
-// (s2, s3) += v: a term of the second word's size.
-__device__ __forceinline__ void ts_add_low(float v, float& s2, float& s3) {
-  const float b = __fadd_rn(s2, v), bb = __fsub_rn(b, s2);
-  s3 = __fadd_rn(s3, __fadd_rn(__fsub_rn(s2, __fsub_rn(b, bb)), __fsub_rn(v, bb)));
-  s2 = b;
-}
-
 // An FP32 value as FP64 and an FP64 value rounded (to nearest even) to FP32,
 // on the integer pipe: a conversion instruction takes a slot of the FP64
 // pipe, as long as some thirty integer operations.  Zeros, subnormals,

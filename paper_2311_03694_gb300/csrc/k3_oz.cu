@@ -338,6 +338,13 @@ __device__ __forceinline__ void oz_sum(const float* __restrict__ D, int64_t M, i
   }
 }
 
+// (s2, s3) += v: a term of the second word's size (beside ts_add).
+__device__ __forceinline__ void ts_add_low(float v, float& s2, float& s3) {
+  const float b = __fadd_rn(s2, v), bb = __fsub_rn(b, s2);
+  s3 = __fadd_rn(s3, __fadd_rn(__fsub_rn(s2, __fsub_rn(b, bb)), __fsub_rn(v, bb)));
+  s2 = b;
+}
+
 // The pairs of one output from k3_tri.cu, [split][hi, lo][bq][M], in split
 // order, in three floats: as double-single sums each split added two roundings of
 // the pair's last bit (n = 1024, r = 512, 64 trajectories, against long double,
