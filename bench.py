@@ -208,6 +208,33 @@ def kernel_traffic(kernel_key):
     return d["bytes_per_launch"] if h.hexdigest() == d["source_sha256"] else None
 
 
+def k3o_faster(n, rank, batch):
+    """Whether the library's rule sends FP64 batches of the skew CP form to K3O (k3o_faster in csrc/grom_internal.h)."""
+    nr = n * rank
+    least = 2 ** 23 if nr >= 2 ** 19 else 3 * 2 ** 22 if nr >= 2 ** 14 else 2 ** 24
+    return nr * batch >= least
+
+
+# -------------------------------------------------------------------- output
+def short_line(line):
+    """The one line printed on stdout: `line` with each result of the wide
+    sections cut to its rate and error (some 4 KB where the whole record has 25,
+    which readers that keep only the tail of the output lose the start of).  The
+    whole record goes to stderr and to --json-out."""
+    def cut(x, keep):
+        return {k: float("%.6g" % v) if isinstance(v, float) else v for k, v in x.items()
+                if any(k.startswith(q) for q in keep) and not isinstance(v, (dict, list))}
+
+    keep = {"variants": ("steps_per_s", "eval_rel_err", "status"), "batched": ("trajectory_steps_per_s", "eval_rel_err"),
+            "fitting": ("s_per_iteration", "solve_ms_per_iteration", "mttkrp_ms")}
+    out = dict(line)
+    for section, names in keep.items():
+        out[section] = {k: cut(v, names) for k, v in (line.get(section) or {}).items()}
+    if line.get("serving"):
+        out["serving"] = cut(line["serving"], ("",))
+    return out
+
+
 # ------------------------------------------------------------------ timing
 def time_steps(torch, tr, steps, stream):
     """ms per step of `steps` steps of an existing trajectory batch (one
@@ -886,7 +913,7 @@ def main():
                                else "k3o (tcgen05 products of %s-bit digit slices; FP64 tolerance)" % (
                                    "7" if n <= 1024 else "6")
                                if storage == "f64" and B >= 16 and (kernel == "tensor" or (
-                                   kernel == "auto" and n * R * B >= (2 ** 23 if n * R >= 2 ** 19 else 3 * 2 ** 22)))
+                                   kernel == "auto" and k3o_faster(n, R, B)))
                                else "k3d project/expand (double-single FP32 GEMMs, FP64 tolerance)"
                                if storage == "f64" and kernel == "auto" and B >= 16
                                else "k3g project/expand (register-tiled FP64 GEMMs)" if B >= 16
@@ -1007,7 +1034,8 @@ def main():
     rom.close()
     if rank_id == 0:
         out = json.dumps(line)
-        print(out)
+        print(out, file=sys.stderr)
+        print(json.dumps(short_line(line)), flush=True)
         if args.json_out:
             with open(args.json_out, "w") as fh:
                 fh.write(out + "\n")
