@@ -24,10 +24,20 @@
 
 #include "ds_arith.cuh"
 #include "grom_internal.h"
+#include "ptx.cuh"
 
 using namespace grom;
 
 constexpr int ALS_PARTS = 256;  // blocks of the residual's reductions
+
+// Of one solve, written by its kernels: whether a pivot broke down, and device
+// clock values in ns at the start and end of the factorisation, of the triangular
+// solves.  (Events around them cost a small fit 2 %: three more records an update
+// on its chain of dependent launches.)
+struct AlsSolve {
+  int bad, pad;
+  unsigned long long f0, f1, s0, s1;
+};
 
 struct grom_als {
   int64_t n = 0, np = 0;
@@ -48,15 +58,15 @@ struct grom_als {
   double* lt = nullptr;                           // L^T
   double* rdiag = nullptr;                        // reciprocals of L's diagonal
   double* part = nullptr;                         // 2 x ALS_PARTS reduction partials
-  int* flag = nullptr;                            // Cholesky breakdown
+  AlsSolve* solve = nullptr;                      // on the device: the last solve's flag and times
   void* k2s = nullptr;
   size_t k2s_bytes = 0;
-  // timing since the last grom_als_stats: device times (CUDA events) of the
-  // tensor-core launches and of the SPD solves (each factorisation from its
-  // first launch, whatever runs beside it, and the triangular solves)
+  // timing since the last grom_als_stats: device times of the tensor-core
+  // launches (CUDA events) and of the SPD solves (each factorisation, whatever
+  // runs beside it, and the triangular solves)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   cudaStream_t side = nullptr;                    // the factorisations' stream
-  cudaEvent_t fork = nullptr, sf0 = nullptr, join = nullptr, sv0 = nullptr, sv1 = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   double mttkrp_ms = 0.0, solve_ms = 0.0;
   int64_t mttkrp_calls = 0;
 };
@@ -174,7 +184,8 @@ __global__ void __launch_bounds__(256) k_gram(const double* __restrict__ F, int6
 
 // H, with the diagonal maximum found by every block (r entries).
 __global__ void k_als_normal(const double* __restrict__ Ga, const double* __restrict__ Gb, int64_t r, double rel,
-                             double* __restrict__ H) {
+                             double* __restrict__ H, AlsSolve* solve) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) solve->f0 = ptx::globaltimer();
   __shared__ double wm[32];
   double m = 0.0;
   for (int64_t a = threadIdx.x; a < r; a += blockDim.x) m = fmax(m, Ga[a * r + a] * Gb[a * r + a]);
@@ -328,11 +339,12 @@ __global__ void __launch_bounds__(UT * UT) k_chol_update(double* H, int64_t r, i
   }
 }
 
-__global__ void k_transpose(const double* __restrict__ L, int64_t r, double* __restrict__ Lt) {
+__global__ void k_transpose(const double* __restrict__ L, int64_t r, double* __restrict__ Lt, AlsSolve* solve) {
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < r * r; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t a = t / r, b = t - a * r;
     Lt[t] = L[b * r + a];
   }
+  if (threadIdx.x == 0) atomicMax(&solve->f1, (unsigned long long)ptx::globaltimer());
 }
 
 // A[i][:] = M[i][:] H^-1 (M given transposed, r x n; H = L L^T): forward
@@ -372,7 +384,8 @@ __device__ __forceinline__ double warp_sum8(double (&v)[SV_T], int lane) {
 
 __global__ void __launch_bounds__(32 * SV_ROWS * SV_WARPS)
     k_als_rowsolve(const double* __restrict__ L, const double* __restrict__ Lt, const double* __restrict__ rdiag,
-                   const double* __restrict__ Mt, int64_t n, int64_t r, double* __restrict__ A) {
+                   const double* __restrict__ Mt, int64_t n, int64_t r, double* __restrict__ A, AlsSolve* solve) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) solve->s0 = ptx::globaltimer();
   extern __shared__ double ybuf[];
   __shared__ double Bs[SV_ROWS][CH][CH + 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, row = w / SV_WARPS, sub = w % SV_WARPS;
@@ -450,6 +463,8 @@ __global__ void __launch_bounds__(32 * SV_ROWS * SV_WARPS)
       row_sync();
     }
   }
+  __syncthreads();
+  if (threadIdx.x == 0) atomicMax(&solve->s1, (unsigned long long)ptx::globaltimer());
 }
 
 // Block b of ALS_PARTS: partial sums of <A, M> (A n x r, M^T r x n) into
@@ -524,7 +539,7 @@ void als_free_fit(grom_als* s) {
     if (p) cudaFree(p), p = nullptr;
   for (double** p : {&s->anew, &s->b1, &s->mt, &s->h, &s->lt, &s->rdiag, &s->part})
     if (*p) cudaFree(*p), *p = nullptr;
-  if (s->flag) cudaFree(s->flag), s->flag = nullptr;
+  if (s->solve) cudaFree(s->solve), s->solve = nullptr;
   if (s->k2s) cudaFree(s->k2s), s->k2s = nullptr;
   s->rcap = 0;
   s->k2s_bytes = 0;
@@ -558,7 +573,7 @@ grom_status als_grow(grom_als* s, int64_t r) {
   if (e == cudaSuccess) e = cudaMalloc(&s->lt, gb);
   if (e == cudaSuccess) e = cudaMalloc(&s->rdiag, (size_t)r * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&s->part, 2 * ALS_PARTS * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&s->flag, sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&s->solve, sizeof(AlsSolve));
   if (e == cudaSuccess) e = cudaMalloc(&s->k2s, need);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -598,11 +613,12 @@ grom_status mttkrp(grom_als* s, int m, int fp, int fq, int64_t r) {
 }
 
 // Waits for the stream; after an MTTKRP its time and the device error word,
-// after a factorisation (ok != nullptr) whether every pivot was positive.
+// after a solve (ok != nullptr) its times and whether every pivot was positive.
 grom_status als_wait(grom_als* s, bool mttkrp_ran, bool* ok) {
-  int flags[2] = {0, 0};
-  GROM_CUDA_TRY(cudaMemcpyAsync(flags, s->err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
-  if (ok) GROM_CUDA_TRY(cudaMemcpyAsync(flags + 1, s->flag, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+  int flags = 0;
+  AlsSolve v{};
+  GROM_CUDA_TRY(cudaMemcpyAsync(&flags, s->err, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
+  if (ok) GROM_CUDA_TRY(cudaMemcpyAsync(&v, s->solve, sizeof(v), cudaMemcpyDeviceToHost, s->stream));
   GROM_CUDA_TRY(cudaStreamSynchronize(s->stream));
   float ms = 0.f;
   if (mttkrp_ran) {
@@ -610,28 +626,31 @@ grom_status als_wait(grom_als* s, bool mttkrp_ran, bool* ok) {
     s->mttkrp_ms += ms;
     ++s->mttkrp_calls;
   }
-  if (flags[0] & DEV_ERR_TIMEOUT) {
+  if (flags & DEV_ERR_TIMEOUT) {
     cudaMemset(s->err, 0, sizeof(int));
     return fail(GROM_ERR_TIMEOUT, "grom_als_fit: a device-side wait timed out");
   }
-  if (ok) *ok = flags[1] == 0;
+  if (ok) {
+    *ok = v.bad == 0;
+    s->solve_ms += 1e-6 * ((double)(v.f1 - v.f0) + (double)(v.s1 - v.s0));
+  }
   return GROM_OK;
 }
 
 // H = Ga o Gb + rel max diag(Ga o Gb) I and its Cholesky factor L (s->h) and
 // L^T (s->lt), on stream st.
 grom_status factorise(grom_als* s, const double* Ga, const double* Gb, int64_t r, double rel, cudaStream_t st) {
-  GROM_CUDA_TRY(cudaMemsetAsync(s->flag, 0, sizeof(int), st));
-  k_als_normal<<<grid_for(r * r), 256, 0, st>>>(Ga, Gb, r, rel, s->h);
+  GROM_CUDA_TRY(cudaMemsetAsync(s->solve, 0, sizeof(AlsSolve), st));
+  k_als_normal<<<grid_for(r * r), 256, 0, st>>>(Ga, Gb, r, rel, s->h, s->solve);
   for (int64_t kb = 0; kb < r; kb += CH) {
-    k_chol_diag<<<1, 128, 0, st>>>(s->h, r, kb, s->rdiag, s->flag);
+    k_chol_diag<<<1, 128, 0, st>>>(s->h, r, kb, s->rdiag, &s->solve->bad);
     if (kb + CH < r) {
       const int64_t rows = r - kb - CH, m = (rows + UT - 1) / UT;
       k_chol_panel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(s->h, r, kb, s->rdiag);
       k_chol_update<<<(unsigned)(m * (m + 1) / 2), UT * UT, 0, st>>>(s->h, r, kb);
     }
   }
-  k_transpose<<<grid_for(r * r), 256, 0, st>>>(s->h, r, s->lt);
+  k_transpose<<<grid_for(r * r), 256, 0, st>>>(s->h, r, s->lt, s->solve);
   GROM_CUDA_TRY(cudaGetLastError());
   return GROM_OK;
 }
@@ -642,7 +661,7 @@ grom_status triangular_solves(grom_als* s, int64_t r, double* dst) {
   if (smem > 12 * 1024)
     GROM_CUDA_TRY(cudaFuncSetAttribute(k_als_rowsolve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   k_als_rowsolve<<<(unsigned)((s->n + SV_ROWS - 1) / SV_ROWS), 32 * SV_ROWS * SV_WARPS, smem, s->stream>>>(
-      s->h, s->lt, s->rdiag, s->mt, s->n, r, dst);
+      s->h, s->lt, s->rdiag, s->mt, s->n, r, dst, s->solve);
   GROM_CUDA_TRY(cudaGetLastError());
   return GROM_OK;
 }
@@ -658,12 +677,10 @@ grom_status ls_update(grom_als* s, int m, int fp, int fq, int64_t r, double ridg
   grom_status st;
   GROM_CUDA_TRY(cudaEventRecord(s->fork, s->stream));
   GROM_CUDA_TRY(cudaStreamWaitEvent(s->side, s->fork, 0));
-  GROM_CUDA_TRY(cudaEventRecord(s->sf0, s->side));
   if ((st = factorise(s, Ga, Gb, r, ridge, s->side))) return st;
   GROM_CUDA_TRY(cudaEventRecord(s->join, s->side));
   if (!have_m && (st = mttkrp(s, m, fp, fq, r))) return st;
   GROM_CUDA_TRY(cudaStreamWaitEvent(s->stream, s->join, 0));
-  GROM_CUDA_TRY(cudaEventRecord(s->sv0, s->stream));
   bool ok = false, ran = !have_m;
   double mu = 0.0;
   for (int attempt = 0; attempt < 4 && !ok; ++attempt) {
@@ -672,16 +689,10 @@ grom_status ls_update(grom_als* s, int m, int fp, int fq, int64_t r, double ridg
       if ((st = factorise(s, Ga, Gb, r, ridge + mu, s->stream))) return st;
     }
     if ((st = triangular_solves(s, r, s->anew))) return st;
-    GROM_CUDA_TRY(cudaEventRecord(s->sv1, s->stream));
     if ((st = als_wait(s, ran, &ok))) return st;
     ran = false;
   }
   if (!ok) return fail(GROM_ERR_INVALID_ARG, "grom_als_fit: a Gram matrix is not positive definite");
-  float ms = 0.f;
-  GROM_CUDA_TRY(cudaEventElapsedTime(&ms, s->sf0, s->join));
-  s->solve_ms += ms;
-  GROM_CUDA_TRY(cudaEventElapsedTime(&ms, s->sv0, s->sv1));
-  s->solve_ms += ms;
   if (dst != s->anew)
     GROM_CUDA_TRY(cudaMemcpyAsync(dst, s->anew, (size_t)(s->n * r) * sizeof(double), cudaMemcpyDeviceToDevice, s->stream));
   return GROM_OK;
@@ -747,9 +758,8 @@ grom_status grom_als_create(int32_t n, const double* tensor, void* stream, grom_
   if (cudaMalloc(&s->err, sizeof(int)) != cudaSuccess || cudaMemsetAsync(s->err, 0, sizeof(int), s->stream) != cudaSuccess)
     return bail(fail(GROM_ERR_OOM, "grom_als_create: device allocation"));
   if (cudaEventCreate(&s->ev0) != cudaSuccess || cudaEventCreate(&s->ev1) != cudaSuccess ||
-      cudaEventCreate(&s->sv0) != cudaSuccess || cudaEventCreate(&s->sv1) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreate(&s->sf0) != cudaSuccess || cudaEventCreate(&s->join) != cudaSuccess ||
+      cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) != cudaSuccess ||
       cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking) != cudaSuccess)
     return bail(cuda_fail(cudaGetLastError(), "grom_als_create: events"));
   // stream the FP64 tensor through a staging buffer by test index
@@ -869,7 +879,7 @@ grom_status grom_als_destroy(grom_als* s) {
   if (!s) return GROM_OK;
   if (s->side) cudaStreamSynchronize(s->side);
   if (s->stream) cudaStreamSynchronize(s->stream);
-  for (cudaEvent_t e : {s->ev0, s->ev1, s->sf0, s->sv0, s->sv1, s->fork, s->join})
+  for (cudaEvent_t e : {s->ev0, s->ev1, s->fork, s->join})
     if (e) cudaEventDestroy(e);
   if (s->side) cudaStreamDestroy(s->side);
   for (auto p : s->x)
