@@ -505,8 +505,9 @@ __global__ void __launch_bounds__(K1T_THREADS, 1) k1t_kernel(const K1TArgs a, co
               double ep, ip;
               int bb;
               // (loaded before the windows, these operands cost the F32X2
-              // stream 2 %: 435 us a step of n = 1024 against 444)
-              step_elem(st, h, n, l, k, i, step_load(st, h, n, l, k, i), v, ep, ip, bb);
+              // stream 2 %: 435 us a step of n = 1024 against 444; loaded
+              // whatever the order, 2 % at n = 1000)
+              step_elem(st, h, n, l, k, i, step_load<false, false>(st, h, n, l, k, i), v, ep, ip, bb);
               ew[b] += ep;
               iw[b] += ip;
               if (bb) {

@@ -62,7 +62,8 @@ __device__ __forceinline__ int step_is_bad(double un) {  // inf or NaN, from the
 struct StepElem {
   double u[3], g[3], hd, mb, ld, f;
 };
-template <bool PLAIN = false>
+// (ALL false: only the ones of order k.)
+template <bool PLAIN = false, bool ALL = true>
 __device__ __forceinline__ StepElem step_load(const StepArgs& a, const double* h, int64_t n, int64_t l, int k,
                                               int64_t i) {
   StepElem x;
@@ -70,8 +71,11 @@ __device__ __forceinline__ StepElem step_load(const StepArgs& a, const double* h
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     const int m = m0 - q < 0 ? m0 - q + 3 : m0 - q;
-    x.u[q] = h[m * n + i];
-    x.g[q] = q == 0 ? 0.0 : h[(3 + m) * n + i];
+    x.u[q] = x.g[q] = 0.0;
+    if (ALL || q < k) {
+      x.u[q] = h[m * n + i];
+      if (q > 0) x.g[q] = h[(3 + m) * n + i];
+    }
   }
   x.hd = a.hdiag[k - 1][i];
   x.mb = !PLAIN && a.mass_diag ? a.mass_diag[i] : 1.0;
