@@ -15,8 +15,9 @@
 // values an output, then their sums) took the time of a step.  Steps of n = R
 // = 1024, FP64 tolerance: 64 trajectories 63.4 -> 49.6 us, 256 177 -> 145,
 // 1024 541 -> 457; n = R = 512, 256 trajectories 80 -> 54.  What bounds it is
-// the L2: a K step of 64 is 192 KB of digits for 2304 columns of products,
-// 7.4 TB/s over the chip, and for small batches the round trip of a tile.
+// the L2: a K step of 64 is 192 KB of digits for 2304 columns of products
+// (projections of 1024 trajectories: 6.4 TB/s there, the tensor pipe 53 % active,
+// cold under ncu), and for small batches the round trip of a tile.
 #include <algorithm>
 
 #include "ds_arith.cuh"
